@@ -88,7 +88,7 @@ static void free_grid(Grid* g) {
   dev_free(g->boxes_d); dev_free(g->gtab); dev_free(g->htab);
   dev_free(g->dtau); dev_free(g->dtauT); dev_free(g->invn);
   free_sources(*g);
-  dev_free(g->geo); dev_free(g->georow); dev_free(g->queue); dev_free(g->err);
+  dev_free(g->geo); dev_free(g->georow); dev_free(g->kap); dev_free(g->queue); dev_free(g->err);
   dev_free(g->cube); dev_free(g->unconv); dev_free(g->xbuf); dev_free(g->xavg);
   dev_free(g->xavg2); dev_free(g->xhi_int); dev_free(g->flags); dev_free(g->counters);
   dev_free(g->bwd_stack); dev_free(g->dq_merged);
@@ -119,18 +119,29 @@ static rt_status ensure_geometry(Grid& g, int mmax) {
   GeoEntry* geo = nullptr;
   GeoRow* georow = nullptr;
   TRY(dev_malloc(&geo, geo_count(mmax) * sizeof(GeoEntry)));
+  const int kmax = std::min(mmax, kKapMax);
+  double* kap = nullptr;
+  double2* binom = nullptr;
   cudaError_t e = dev_malloc(&georow, georow_count(mmax) * sizeof(GeoRow));
-  if (e == cudaSuccess) e = launch_geometry(geo, georow, mmax, g.stream);
+  if (e == cudaSuccess) e = dev_malloc(&kap, 2 * georow_count(kmax) * sizeof(double));
+  if (e == cudaSuccess) e = dev_malloc(&binom, (size_t)(kmax + 1) * (kmax + 2) / 2 * sizeof(double2));
+  if (e == cudaSuccess) e = launch_geometry(geo, georow, kap, binom, mmax, g.stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(g.stream);  // binom is still read
+  dev_free(binom);
   if (e != cudaSuccess) {
     dev_free(geo);
     dev_free(georow);
+    dev_free(kap);
     return cuda_fail(e, "geometry");
   }
   dev_free(g.geo);
   dev_free(g.georow);
+  dev_free(g.kap);
   g.geo = geo;
   g.georow = georow;
+  g.kap = kap;
   g.geo_mmax = mmax;
+  g.kap_mmax = kmax;
   return RT_OK;
 }
 
@@ -148,6 +159,7 @@ static TraceArgs base_args(Grid& g) {
   a.dtau = g.dtau;
   a.dtauT = g.dtauT;
   a.invn = g.invn;
+  a.thick = g.invn;
   a.src = g.src;
   a.ndot = g.ndot;
   a.r2lim = g.r2lim;
@@ -160,12 +172,18 @@ static TraceArgs base_args(Grid& g) {
   a.rtab_hcap = g.rtab_hcap;
   a.rtab_slot = g.rtab_slot;
   a.rtab_max_r2 = g.rtab_max_r2;
+  a.rtab_lay = g.rtab_lay;
+  a.ftab = g.ftab;
+  a.ftab_lay = g.ftab_lay;
   a.itab = g.itab;
   a.itab_off = g.itab_off;
   a.neg_zero = -0.0;
   a.interp_mode = g.interp_mode;
   a.tau_w0 = g.tau_w0;
   a.geo_mmax = g.geo_mmax;
+  a.kap = g.kap;
+  a.kap_mmax = g.kap_mmax;
+  a.kappa = g.kap ? g.kap + georow_count(g.kap_mmax) : nullptr;
   a.tab.g = g.gtab;
   a.tab.h = g.htab;
   a.tab.kind = g.tab_kind;
@@ -218,6 +236,132 @@ static rt_status check_ready(Grid& g, const char* who) {
   return RT_OK;
 }
 
+// Scratch cubes of the plain schedule for nsrc sources.
+constexpr int kPlainBlock = 256;
+static rt_status ensure_cube(Grid& g, int nsrc, int* out_grid, int* out_E) {
+  const int E = std::max(1, std::min(isqrt_h(g.max_r2), g.nmax / 2));
+  const int grid = std::min(nsrc, std::max(1, shells_max_grid(kPlainBlock)));
+  const size_t side = 2 * (size_t)E + 1;
+  const size_t need = side * side * side * sizeof(double) * (size_t)grid;
+  if (need > g.cube_bytes) {
+    dev_free(g.cube);
+    g.cube = nullptr;
+    g.cube_bytes = 0;
+    TRY(dev_malloc(&g.cube, need));
+    g.cube_bytes = need;
+  }
+  *out_grid = grid;
+  *out_E = E;
+  return RT_OK;
+}
+
+// Whether the batched rates go to rates.cu (its precompute: zeros for the thick terms).
+static bool takes_rates_kernels(const Grid& g) { return g.interp_mode == RT_INTERP_GEOMETRIC; }
+
+// First source (LPT order) whose layers fit half-width hlim; ns: none.
+static int first_fitting(const Grid& g, const int* r2s, int ns, int hlim) {
+  if (hlim <= 0) return ns;
+  int lo = 0, hi = ns;
+  while (lo < hi) {
+    const int mid = (lo + hi) / 2;
+    if (face_hcap(r2s[mid], g.nmax) <= hlim) hi = mid; else lo = mid + 1;
+  }
+  return lo;
+}
+
+// Launches of the batched rates: sources [cut[k], cut[k+1]) (LPT order) by CTAs of
+// mode[0] threads (k = 0) or by warps with one quadrant, two, or a whole face (k = 1..3).
+struct RatesPlan {
+  int mode[4] = {128, 1, 2, 4};
+  int cut[5] = {0, 0, 0, 0, 0};
+};
+
+// With rt_set_schedule (or an autotuned choice): its thresholds.  Otherwise by rule.
+// Measured on uniform catalogues (batched trace, ms: CTA of 128 / one quadrant per warp
+// / two / a face; 128^3): R = 12 (half-width 8), 4e4 sources 16.7 / 10.4 / 7.3 / 5.2;
+// R = 22 (15), 1e4: 7.4 / 4.7 / 4.0 / 3.7; R = 27 (19), 8e3: 7.7 / 5.1 / 4.7 / 5.8;
+// R = 33 (23), 5e3: 6.5 / 4.8 / 4.6 / -; R = 50 (35), 2e3: 5.8 / 5.3 / 7.0 / -; R = 60
+// (42), 1e3: 4.8 / 5.3 / - / -: hence the half-widths.  A launch pays for its last
+// wave, so where several classes would be launched a class of few items joins the finer
+// one before it (64^3, 1e3 sources of R = 5..50: one launch 0.52, three 0.87 ms), and
+// where one quadrant would take a warp longer than all work takes the GPU, CTAs trace
+// everything (64^3, 10 sources of R = 20: 0.048 against 0.057 ms; 128^3, 40 of R = 40:
+// 0.123 / 0.187), of 256 threads where not even every SM gets two.
+static RatesPlan rates_plan(const Grid& g, const int* r2s, int ns) {
+  RatesPlan p;
+  p.mode[0] = g.block_big;
+  p.cut[4] = ns;
+  if (g.explicit_schedule) {
+    p.cut[1] = first_fitting(g, r2s, ns, g.hsmall);
+    p.cut[2] = p.cut[3] = g.ftab ? std::max(p.cut[1], first_fitting(g, r2s, ns, g.hface)) : ns;
+    return p;
+  }
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const double warps = 16.0 * sms;  // resident at the larger half-widths
+  const double r = std::sqrt((double)r2s[0]);
+  const double ball = std::min(4.18879 * r * r * r, (double)g.nmax * g.nmax * g.nmax);
+  p.mode[0] = 128;
+  if (ball * warps > 1.2 * 24 * (double)g.source_voxels) {
+    if (24 * ns <= 2 * sms && face_hcap(r2s[0], g.nmax) >= 24) p.mode[0] = 256;
+    p.cut[1] = p.cut[2] = p.cut[3] = ns;
+    return p;
+  }
+  const int lim[4] = {0, 38, 23, g.ftab ? 16 : 0};
+  for (int k = 1; k < 4; ++k) p.cut[k] = std::max(p.cut[k - 1], first_fitting(g, r2s, ns, lim[k]));
+  for (int k = 3; k > 1; --k) {
+    const double items = 24.0 / p.mode[k] * (p.cut[k + 1] - p.cut[k]);
+    if (items < (p.cut[k] > 0 ? 6 : 1.2) * warps) p.cut[k] = p.cut[k + 1];
+  }
+  return p;
+}
+
+static rt_status run_rates(Grid& g, const TraceArgs& a, const int* items, int ns) {
+  const int* r2s = g.r2_sorted_h.data();
+  const RatesPlan plan = rates_plan(g, r2s, ns);
+  const int *mode = plan.mode, *cut = plan.cut;
+  TRY(cudaMemsetAsync(g.queue, 0, 4 * sizeof(int), g.stream));
+  for (int k = 0; k < 4; ++k) {
+    if (cut[k + 1] <= cut[k]) continue;
+    TraceArgs b = a;
+    b.items = items;
+    b.hcap = face_hcap(r2s[cut[k]], g.nmax);
+    const int per = k == 0 ? 24 : 24 / mode[k];
+    b.item_begin = per * cut[k];
+    b.n_items = per * cut[k + 1];
+    b.queue = g.queue + k;
+    const size_t smem = rates_smem_bytes(b.hcap, mode[k]);
+    if (smem > 227 * 1024)
+      return fail(RT_ERR_INVALID, "rt_raytrace: radius too large for the batched schedule's "
+                                  "shared-memory layers; use RT_SCHED_PLAIN");
+    int wpb = 1, maxg = 0;
+    if (k == 0) {
+      maxg = rates_max_grid(mode[k], smem, 1, a.early_exit != 0);
+    } else {
+      // CTAs of 1..8 warps, whichever keeps the most warps resident (a warp's shared
+      // memory grows with its layer capacity, and every CTA also reserves some; ties
+      // go to the larger CTA)
+      for (int cand = 8; cand >= 1; --cand) {
+        const int mg = rates_max_grid(mode[k], smem * cand, cand, a.early_exit != 0);
+        if (mg * cand > maxg * wpb) {
+          maxg = mg;
+          wpb = cand;
+        }
+      }
+    }
+    if (maxg <= 0) return fail(RT_ERR_CUDA, "rt_raytrace: no occupancy for a rate kernel");
+    const int nitem = b.n_items - b.item_begin;
+    const int grid = std::max(1, std::min((nitem + wpb - 1) / wpb, maxg));
+    TRY(launch_rates(g, b, mode[k], grid, smem * wpb, wpb));
+    if (++g.stats.launches == 1) {
+      g.stats.block = k == 0 ? mode[k] : 32 * wpb;
+      g.stats.grid = grid;
+    }
+  }
+  return RT_OK;
+}
+
 // Trace all sources, adding rates into `gamma` (already zeroed) or writing one
 // source's column densities.  `items`/`n_items` select the work.
 // single_r2 >= 0: the items are the 24 of one source with that R^2 limit (else
@@ -232,19 +376,16 @@ static rt_status run_trace(Grid& g, double* gamma, double* coldens, const int* i
   a.early_exit = early_exit ? 1 : 0;
   g.stats.launches = 0;
   TRY(cudaMemsetAsync(g.counters, 0, sizeof(unsigned long long), g.stream));
+  const bool od = a.interp_mode == RT_INTERP_OPTICAL_DEPTH;
+  const bool rates = gamma && takes_rates_kernels(g);
+  if (schedule != RT_SCHED_PLAIN && g.nmax > 1290)
+    return fail(RT_ERR_INVALID, "rt_raytrace: the batched schedule needs boxes of at most "
+                                "1290^3 cells (32-bit offsets); use RT_SCHED_PLAIN");
   if (schedule == RT_SCHED_PLAIN) {
-    const int E = std::max(1, std::min(isqrt_h(g.max_r2), g.nmax / 2));
-    const int block = 256;
-    int grid = std::min(nsrc_plain, std::max(1, shells_max_grid(block)));
-    const size_t side = 2 * (size_t)E + 1;
-    const size_t need = side * side * side * sizeof(double) * (size_t)grid;
-    if (need > g.cube_bytes) {
-      dev_free(g.cube);
-      g.cube = nullptr;
-      g.cube_bytes = 0;
-      TRY(dev_malloc(&g.cube, need));
-      g.cube_bytes = need;
-    }
+    const int block = kPlainBlock;
+    int grid = 0, E = 0;
+    rt_status cs = ensure_cube(g, nsrc_plain, &grid, &E);
+    if (cs != RT_OK) return cs;
     a.scratch = g.cube;
     a.hcap = E;
     a.items = items;
@@ -255,10 +396,12 @@ static rt_status run_trace(Grid& g, double* gamma, double* coldens, const int* i
     g.stats.grid = grid;
     g.stats.launches = 1;
     g.stats.items = nsrc_plain;
+  } else if (rates) {
+    rt_status rs = run_rates(g, a, items, n_items / 24);
+    if (rs != RT_OK) return rs;
+    TRY(launch_add_thick(g, gamma, skip));
+    g.stats.items = n_items;
   } else {
-    if (g.nmax > 1290)
-      return fail(RT_ERR_INVALID, "rt_raytrace: the batched schedule needs boxes of at most "
-                                  "1290^3 cells (32-bit offsets); use RT_SCHED_PLAIN");
     // Batched: items of large sources are traced by whole CTAs, items whose
     // layers fit g.hsmall by single warps, and the faces of sources whose layers
     // fit g.hface by single warps that trace a face whole.  Items come
@@ -266,19 +409,9 @@ static rt_status run_trace(Grid& g, double* gamma, double* coldens, const int* i
     // contiguous range of sources: [0, pw) CTAs, [pw, p4) warps, [p4, ns) whole faces.
     const int* r2s = single_r2 >= 0 ? &single_r2 : g.r2_sorted_h.data();
     const int ns = n_items / 24;
-    auto first_fitting = [&](int hlim) {  // first source whose layers fit hlim (ns: none)
-      if (hlim <= 0) return ns;
-      int lo = 0, hi = ns;
-      while (lo < hi) {
-        const int mid = (lo + hi) / 2;
-        if (face_hcap(r2s[mid], g.nmax) <= hlim) hi = mid; else lo = mid + 1;
-      }
-      return lo;
-    };
-    const int pw = first_fitting(g.hsmall);
-    const int p4 = std::max(pw, first_fitting(g.hface));
+    const int pw = first_fitting(g, r2s, ns, g.hsmall);
+    const int p4 = std::max(pw, first_fitting(g, r2s, ns, g.hface));
     const int hbig = face_hcap(r2s[0], g.nmax);
-    const bool od = a.interp_mode == RT_INTERP_OPTICAL_DEPTH;
     TRY(cudaMemsetAsync(g.queue, 0, 3 * sizeof(int), g.stream));
     a.items = items;
     g.stats.launches = 0;
@@ -286,9 +419,10 @@ static rt_status run_trace(Grid& g, double* gamma, double* coldens, const int* i
     // warp's shared memory grows with its layer capacity, and every CTA also
     // reserves some; ties go to the larger CTA)
     auto warp_launch = [&](int mode, int hcap, int item_begin, int item_end, int* queue) {
+      const size_t smem = faces_smem_bytes(hcap, mode, od);
       int wpb = 8, maxg = 0;
       for (int cand = 8; cand >= 1; --cand) {
-        const int mg = faces_max_grid(mode, faces_smem_bytes(hcap, mode, od) * cand, cand, od);
+        const int mg = faces_max_grid(mode, smem * cand, cand, od);
         if (mg * cand > maxg * wpb) {
           maxg = mg;
           wpb = cand;
@@ -303,7 +437,7 @@ static rt_status run_trace(Grid& g, double* gamma, double* coldens, const int* i
       b.queue = queue;
       const int nitem = item_end - item_begin;
       const int grid = std::max(1, std::min((nitem + wpb - 1) / wpb, maxg));
-      TRY(launch_trace_faces(g, b, mode, grid, faces_smem_bytes(hcap, mode, od) * wpb, wpb));
+      TRY(launch_trace_faces(g, b, mode, grid, smem * wpb, wpb));
       g.stats.launches += 1;
       if (g.stats.launches == 1) {
         g.stats.block = 32 * wpb;
@@ -554,11 +688,11 @@ rt_status rt_raytrace(rt_grid_t h, double* d_gamma, int schedule) {
   Grid& g = *reinterpret_cast<Grid*>(h);
   rt_status st = check_ready(g, "rt_raytrace");
   if (st != RT_OK) return st;
+  if (schedule == RT_SCHED_AUTO) schedule = g.auto_plain ? RT_SCHED_PLAIN : RT_SCHED_BATCHED;
   TRY(cudaEventRecord(g.ev[0], g.stream));
-  TRY(launch_precompute(g));
+  TRY(launch_precompute(g, schedule != RT_SCHED_PLAIN && takes_rates_kernels(g)));
   TRY(cudaMemsetAsync(d_gamma, 0, g.ncell * sizeof(double), g.stream));
   TRY(cudaEventRecord(g.ev[1], g.stream));
-  if (schedule == RT_SCHED_AUTO) schedule = g.auto_plain ? RT_SCHED_PLAIN : RT_SCHED_BATCHED;
   if (g.nsrc > 0) {
     if (schedule == RT_SCHED_PLAIN)
       st = run_trace(g, d_gamma, nullptr, nullptr, g.nsrc, RT_SCHED_PLAIN, g.nsrc);
@@ -589,7 +723,7 @@ rt_status rt_raytrace_source_coldens(rt_grid_t h, int src, double* d_coldens, in
   int hitems[24];
   for (int q = 0; q < 24; ++q) hitems[q] = (p << 5) | q;
   TRY(cudaMemcpyAsync(g.queue + 8, hitems, 24 * sizeof(int), cudaMemcpyHostToDevice, g.stream));
-  TRY(launch_precompute(g));
+  TRY(launch_precompute(g, false));
   TRY(cudaMemsetAsync(d_coldens, 0, g.ncell * sizeof(double), g.stream));
   if (schedule == RT_SCHED_PLAIN) {
     hitems[0] = p;
@@ -616,7 +750,7 @@ rt_status rt_get_stats(rt_grid_t h, rt_stats* out) {
   TRY(cudaMemcpy(&rc, g.counters, sizeof(rc), cudaMemcpyDeviceToHost));
   g.stats.rate_cells = (int64_t)rc;
   g.stats.kernel_launches = g_launches.load();
-  g.stats.row_table_bytes = g.rtab ? g.rtab_bytes + g.itab_bytes : 0;
+  g.stats.row_table_bytes = g.rtab ? g.rtab_bytes + g.itab_bytes + g.ftab_bytes : 0;
   *out = g.stats;
   return latched_errors(g);
 }
@@ -700,7 +834,7 @@ rt_status rt_iterate(rt_grid_t h, double* d_x, double dt_s, double alpha_H, doub
     double* xin = (k % 2 == 0) ? g.xavg : g.xavg2;
     double* xout = (k % 2 == 0) ? g.xavg2 : g.xavg;
     TRY(launch_one_minus(xin, g.xhi_int, g.ncell, skip, g.stream));
-    TRY(launch_precompute(g, skip));
+    TRY(launch_precompute(g, takes_rates_kernels(g), skip));
     TRY(launch_zero(d_gamma, g.ncell, skip, g.stream));
     TRY(cudaMemsetAsync(g.unconv, 0, sizeof(int64_t), g.stream));
     if (g.nsrc > 0) {
@@ -792,7 +926,7 @@ rt_status rt_raytrace_backward(rt_grid_t h, const double* d_dL_dgamma, double* d
   if (g.interp_mode != RT_INTERP_GEOMETRIC)
     return fail(RT_ERR_INVALID, "rt_raytrace_backward: the adjoint is built for the geometric "
                                 "weights (rt_set_interpolation mode 0)");
-  TRY(launch_precompute(g));
+  TRY(launch_precompute(g, false));
   TRY(cudaMemsetAsync(d_dL_dlog_nHI, 0, g.ncell * sizeof(double), g.stream));
   if (g.nsrc == 0) return RT_OK;
   if (g.dq_cap < g.nsrc) {
@@ -916,6 +1050,7 @@ rt_status rt_set_schedule(rt_grid_t h, int block_big, int hsmall, int hface) {
   g.block_big = block_big;
   g.hsmall = hsmall;
   g.hface = hface;
+  g.explicit_schedule = true;
   ++g.epoch;
   return RT_OK;
 }
@@ -951,12 +1086,14 @@ rt_status rt_autotune(rt_grid_t h, const char* cache_path, int* h_block, int* h_
       std::istringstream ls(line);
       std::string k;
       int b = 0, hs = -1, hf = -1, ap = -1;
+      std::string how;
       if ((ls >> k >> b >> hs >> hf >> ap) && k == key && (b == 128 || b == 256) && hs >= 0 &&
           hs <= 32 && hf >= 0 && hf <= 20 && (ap == 0 || ap == 1)) {
         g.block_big = b;
         g.hsmall = hs;
         g.hface = hf;
         g.auto_plain = ap;
+        g.explicit_schedule = !((ls >> how) && how == "rule");
         report();
         return RT_OK;
       }
@@ -987,8 +1124,13 @@ rt_status rt_autotune(rt_grid_t h, const char* cache_path, int* h_block, int* h_
   const int blocks[] = {128, 256};
   const int hss[] = {0, 11, 15, 19, 22, 24, 27, 30};
   const int hfs[] = {9, 11, 13, 15, 17, 19};
-  float best = 1e30f;
+  // stage 0: the rule on sizes (rates.cu's kernels only), kept unless thresholds beat it
+  float best = 1e30f, rule = 1e30f;
   int bb = g.block_big, bh = g.hsmall, bf = 0;
+  const bool was_explicit = g.explicit_schedule;
+  g.explicit_schedule = false;
+  if (takes_rates_kernels(g)) timed(rule);
+  g.explicit_schedule = true;
   g.hface = 0;
   for (int b : blocks)
     for (int hs : hss) {
@@ -1036,8 +1178,18 @@ rt_status rt_autotune(rt_grid_t h, const char* cache_path, int* h_block, int* h_
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   dev_free(gam);
-  if (st != RT_OK) return st;
+  if (st != RT_OK) {
+    g.explicit_schedule = was_explicit;
+    return st;
+  }
   g.hface = bf;
+  if (rule <= best) {  // reported as the closest thresholds
+    best = rule;
+    g.explicit_schedule = false;
+    g.block_big = bb = 128;
+    g.hsmall = bh = 32;
+    g.hface = bf = 16;
+  }
   // stage 3: the paper's block-per-source schedule against the tuned batched one
   // (RT_SCHED_AUTO then takes the faster)
   if (st == RT_OK) {
@@ -1059,7 +1211,8 @@ rt_status rt_autotune(rt_grid_t h, const char* cache_path, int* h_block, int* h_
   report();
   if (cache_path) {
     std::ofstream out(cache_path, std::ios::app);
-    out << key << " " << bb << " " << bh << " " << bf << " " << g.auto_plain << "\n";
+    out << key << " " << bb << " " << bh << " " << bf << " " << g.auto_plain
+        << (g.explicit_schedule ? "" : " rule") << "\n";
   }
   return RT_OK;
 }

@@ -45,16 +45,26 @@ inline int64_t geo_count(int mmax) { return geo_index(mmax + 1, 0, 0); }
 
 // Row-major geometry for the batched trace: entry (m, a1, a2), 0 <= a1, a2 <= m,
 // holds the weights in the cell's own orientation (a = a1/m, b = a2/m):
-//   w1 = (1-a)(1-b), w2 = a(1-b), w3 = (1-a)b, w4 = ab, ds = sqrt(1 + (a1^2+a2^2)/m^2)
+//   w1 = (1-a)(1-b), w2 = a(1-b), w3 = (1-a)b, w4 = ab, ds = sqrt(1 + (a1^2+a2^2)/m^2),
+//   invv, thin as in GeoEntry
 // (bit-identical to the (lo, hi) table's values; consecutive a2 are adjacent).
 struct __align__(16) GeoRow {
   double w1, w2, w3, w4;
-  double ds, pad;
+  double ds, pad, invv, thin;
 };
 __host__ __device__ inline int64_t georow_index(int m, int a1, int a2) {
   return (int64_t)m * (m + 1) * (2 * m + 1) / 6 - 1 + (int64_t)a1 * (m + 1) + a2;
 }
 inline int64_t georow_count(int mmax) { return georow_index(mmax + 1, 0, 0); }
+
+// kappa = C(m, a1) C(m, a2) and kappa ds for the batched rates (rates.cu), at
+// georow_index(m, a1, a2), for layers m <= kKapMax (no layer that the batched
+// schedule's shared memory holds lies beyond 170; kappa < 2^(2m)).
+constexpr int kKapMax = 200;
+
+// Largest layer half-width with face tables (the largest that rt_set_schedule accepts
+// for whole faces).
+constexpr int kFaceHcap = 20;
 
 // Rate tables on the device.
 struct TabDev {
@@ -71,6 +81,7 @@ struct TraceArgs {
   const double* dtau;    // sigma0*cell*n_H*x_HI, C order per box
   const double* dtauT;   // the same, axes rotated to (k, i, j) per box
   const double* invn;    // 1/(n_H x_HI)
+  double* thick;         // rates.cu: sum of the thick terms, without the factor 1/n_HI
   double* gamma;         // output rates (may be null)
   double* coldens;       // optional per-source column density output
   const SrcDev* src;
@@ -83,6 +94,9 @@ struct TraceArgs {
   const GeoEntry* geo;
   const GeoRow* georow;
   int geo_mmax;
+  const double* kap;     // kappa ds (rates.cu)
+  const double* kappa;
+  int kap_mmax;
   TabDev tab;
   double tau_lim;
   double sigma0;
@@ -106,6 +120,9 @@ struct TraceArgs {
   const int* rtab_hcap;   // largest layer half-width of each R^2 limit
   const int* rtab_slot;   // R^2 limit -> slot, for 0..rtab_max_r2
   int rtab_max_r2;        // -1: no tables
+  const int4* rtab_lay;   // per blob: offset, bytes, cells, half-width of the layer
+  const unsigned char* ftab;  // face tables (rates.cu) of the limits up to kFaceHcap
+  const int4* ftab_lay;       // the same for them, at the same entries
   // Interior row tables of the same (R^2 limit, m) layers, for faces traced
   // whole (see k_interior_tables): blob of layer m at itab + itab_off[same index].
   const unsigned char* itab;
@@ -143,7 +160,7 @@ struct Grid {
   // derived per-cell fields (owned)
   double* dtau = nullptr;
   double* dtauT = nullptr;
-  double* invn = nullptr;
+  double* invn = nullptr;  // 1/n_HI, or the thick terms' sum of the batched rates
 
   // sources (owned, ingested)
   int nsrc_in = 0;         // as given
@@ -183,6 +200,10 @@ struct Grid {
   int* rtab_first = nullptr;
   int* rtab_hcap = nullptr;
   int* rtab_slot = nullptr;
+  int4* rtab_lay = nullptr;
+  unsigned char* ftab = nullptr;
+  int4* ftab_lay = nullptr;
+  int64_t ftab_bytes = 0;
   int rtab_max_r2 = -1;
   int rtab_mcap = 0;
   int64_t rtab_bytes = 0;
@@ -195,6 +216,8 @@ struct Grid {
   GeoEntry* geo = nullptr;
   GeoRow* georow = nullptr;
   int geo_mmax = 0;
+  double* kap = nullptr;  // kappa ds, then kappa, of the layers up to kap_mmax
+  int kap_mmax = 0;
 
   // scratch
   int* queue = nullptr;
@@ -210,6 +233,7 @@ struct Grid {
   int block_big = 128;      // threads per CTA for large-source items
   int hsmall = 19;          // items whose layers fit this half-width run one per warp
   int hface = 13;           // ... and those fitting this one whole faces per warp
+  bool explicit_schedule = false;  // by rt_set_schedule or the autotuner; else by rule
   int auto_plain = 0;       // RT_SCHED_AUTO takes the plain schedule (autotuner's choice)
   int warps_per_block = 8;  // warp-mode CTA size of the last trace (1..8 warps)
   unsigned long long* counters = nullptr;  // [0]: rate evaluations of the last trace
@@ -273,10 +297,14 @@ rt_status fail(rt_status st, const std::string& msg);
 rt_status cuda_fail(cudaError_t e, const char* what);
 
 // launchers (defined in the kernel translation units)
-cudaError_t launch_precompute(Grid& g, const int* skip = nullptr);
+// dtau, its rotated copy, and 1/n_HI or (for the batched rates: thick) zeros in g.invn
+cudaError_t launch_precompute(Grid& g, bool thick, const int* skip = nullptr);
+// gamma += thick / n_HI where thick != 0
+cudaError_t launch_add_thick(Grid& g, double* gamma, const int* skip);
 cudaError_t launch_zero(double* p, int64_t n, const int* skip, cudaStream_t s);
 cudaError_t launch_validate_fields(Grid& g, const double* nH, const double* xHI);
-cudaError_t launch_geometry(GeoEntry* geo, GeoRow* georow, int mmax, cudaStream_t s);
+cudaError_t launch_geometry(GeoEntry* geo, GeoRow* georow, double* kap, double2* binom, int mmax,
+                            cudaStream_t s);
 cudaError_t launch_trace_faces(Grid& g, const TraceArgs& a, int block, int grid, size_t smem,
                                int wpb = 8);  // wpb: warps per CTA in warp mode (block 32)
 cudaError_t launch_trace_shells(Grid& g, const TraceArgs& a, int block, int grid);
@@ -284,6 +312,11 @@ cudaError_t launch_trace_shells(Grid& g, const TraceArgs& a, int block, int grid
 size_t faces_smem_bytes(int hcap, int block, bool od = false);
 int faces_max_grid(int block, size_t smem, int wpb = 8, bool od = false);
 int shells_max_grid(int block);
+// batched rates with the geometric weights (rates.cu); mode: quadrants per warp (1, 2)
+// or 4 for whole faces (wpb warps per CTA), or threads of a CTA (128, 256)
+cudaError_t launch_rates(Grid& g, const TraceArgs& a, int mode, int grid, size_t smem, int wpb);
+size_t rates_smem_bytes(int hcap, int mode);  // per CTA (warp modes: per warp)
+int rates_max_grid(int mode, size_t smem, int wpb, bool exit);
 rt_status ingest_sources(Grid& g, int nsrc, const int32_t* d_pos, const int32_t* d_box,
                          const double* d_ndot, const double* d_radius);
 cudaError_t launch_chemistry(Grid& g, const double* gamma, const double* x0, const double* xavg_in,

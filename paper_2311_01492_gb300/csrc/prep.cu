@@ -45,7 +45,10 @@ cudaError_t launch_validate_fields(Grid& g, const double* nH, const double* xHI)
 // copy dtauT[k][i][j] so that the z faces read rows of constant k contiguously.
 // n_H is the proper density: the given (comoving) one times inv_a3 = a^-3 in an
 // expanding background (inv_a3 = 1 otherwise, an exact no-op); cell (in the
-// box records) is the proper cell size.
+// box records) is the proper cell size.  THICK: zeros instead of 1/n_HI (the batched
+// rates divide their summed thick terms by n_HI once per cell, k_add_thick; an FP64
+// division per cell made this kernel 2.4 times its memory time at 250^3).
+template <bool THICK>
 __global__ void k_precompute(const BoxDev* __restrict__ boxes, const double* __restrict__ nH,
                              const double* __restrict__ xHI, double inv_a3,
                              double* __restrict__ dtau, double* __restrict__ dtauT,
@@ -67,7 +70,7 @@ __global__ void k_precompute(const BoxDev* __restrict__ boxes, const double* __r
         const double nh = nH[idx] * inv_a3, x = xHI[idx];
         const double d = (B.sig_cell * nh) * x;
         dtau[idx] = d;
-        invn[idx] = 1.0 / (nh * x);
+        invn[idx] = THICK ? 0.0 : 1.0 / (nh * x);
         tile[yy][tx] = d;
       }
     }
@@ -81,11 +84,34 @@ __global__ void k_precompute(const BoxDev* __restrict__ boxes, const double* __r
   }
 }
 
-cudaError_t launch_precompute(Grid& g, const int* skip) {
+cudaError_t launch_precompute(Grid& g, bool thick, const int* skip) {
   const int n = g.nmax;
   dim3 grid((n + 31) / 32, (unsigned)std::min<int64_t>(((int64_t)n * n + 31) / 32, 65535), g.nbox);
-  k_precompute<<<grid, dim3(32, 8), 0, g.stream>>>(g.boxes_d, g.nH, g.xHI, g.inv_a3, g.dtau,
-                                                    g.dtauT, g.invn, skip);
+  if (thick)
+    k_precompute<true><<<grid, dim3(32, 8), 0, g.stream>>>(g.boxes_d, g.nH, g.xHI, g.inv_a3, g.dtau,
+                                                           g.dtauT, g.invn, skip);
+  else
+    k_precompute<false><<<grid, dim3(32, 8), 0, g.stream>>>(g.boxes_d, g.nH, g.xHI, g.inv_a3, g.dtau,
+                                                            g.dtauT, g.invn, skip);
+  count_launch();
+  return cudaGetLastError();
+}
+
+// gamma += thick / n_HI (Eq. sugg's 1/n_HI, taken out of the sum over sources)
+__global__ void k_add_thick(int64_t n, const double* __restrict__ nH, const double* __restrict__ xHI,
+                            double inv_a3, const double* __restrict__ thick,
+                            double* __restrict__ gamma, const int* __restrict__ skip) {
+  if (skip && *skip) return;
+  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n;
+       c += (int64_t)gridDim.x * blockDim.x) {
+    const double t = thick[c];
+    if (t != 0.0) gamma[c] += t / ((nH[c] * inv_a3) * xHI[c]);
+  }
+}
+
+cudaError_t launch_add_thick(Grid& g, double* gamma, const int* skip) {
+  const int grid = (int)std::min<int64_t>((g.ncell + 255) / 256, 152 * 16);
+  k_add_thick<<<grid, 256, 0, g.stream>>>(g.ncell, g.nH, g.xHI, g.inv_a3, g.invn, gamma, skip);
   count_launch();
   return cudaGetLastError();
 }
@@ -108,6 +134,38 @@ cudaError_t launch_zero(double* p, int64_t n, const int* skip, cudaStream_t s) {
 // Entry (m, lo, hi): bilinear weights of Sec. 3.1 for a = lo/m, b = hi/m and
 // the path length ds = sqrt(1 + (lo^2+hi^2)/m^2).  Both are computed with
 // correctly rounded IEEE division and square root.
+// Binomial coefficients C(m, a), a <= m <= kKapMax, at m (m + 1) / 2 + a as the sum
+// of two doubles: they grow to 2^(2m), and the products of two are rounded only once
+// when they enter kappa and kappa ds.  C(m, a) = C(m, a-1) (m - a + 1) / a.
+__global__ void k_binomials(double2* __restrict__ b, int mmax) {
+  const int m = blockIdx.x;
+  if (m > mmax) return;
+  for (int a = threadIdx.x; a <= m; a += blockDim.x) {
+    double hi = 1.0, lo = 0.0;
+    const int k = min(a, m - a);
+    for (int i = 1; i <= k; ++i) {
+      const double x = (double)(m - i + 1), y = (double)i;
+      double ph = hi * x;
+      double pl = fma(hi, x, -ph) + lo * x;
+      const double q = (ph + pl) / y;
+      const double r = fma(-q, y, ph) + pl;
+      const double q2 = r / y;
+      hi = q + q2;
+      lo = q2 - (hi - q);
+    }
+    b[m * (m + 1) / 2 + a] = make_double2(hi, lo);
+  }
+}
+
+// kappa = C(m, a1) C(m, a2) as the sum of two doubles
+__device__ __forceinline__ double2 kappa_dd(const double2* __restrict__ b, int m, int a1, int a2) {
+  const double2 x = b[m * (m + 1) / 2 + a1], y = b[m * (m + 1) / 2 + a2];
+  const double ph = x.x * y.x;
+  const double pl = fma(x.x, y.x, -ph) + (x.x * y.y + x.y * y.x);
+  const double hi = ph + pl;
+  return make_double2(hi, pl - (hi - ph));
+}
+
 __global__ void k_geometry(GeoEntry* __restrict__ geo, int mmax) {
   const int m = blockIdx.x + 1;
   if (m > mmax) return;
@@ -135,7 +193,8 @@ __global__ void k_geometry(GeoEntry* __restrict__ geo, int mmax) {
 }
 
 // Row-major entry (m, a1, a2) with the same correctly rounded expressions.
-__global__ void k_geometry_rows(GeoRow* __restrict__ geo, int mmax) {
+__global__ void k_geometry_rows(GeoRow* __restrict__ geo, double* __restrict__ kap,
+                                double* __restrict__ kappa, const double2* __restrict__ binom, int mmax) {
   const int m = blockIdx.x + 1;
   if (m > mmax) return;
   const int cnt = (m + 1) * (m + 1);
@@ -150,13 +209,28 @@ __global__ void k_geometry_rows(GeoRow* __restrict__ geo, int mmax) {
     e.w4 = x * y;
     e.ds = sqrt(1.0 + (double)(a1 * a1 + a2 * a2) / (double)(m * m));
     e.pad = 0.0;
+    const double r2 = (double)(m * m + a1 * a1 + a2 * a2);
+    const double fourpi = 12.566370614359172;
+    e.invv = 1.0 / (fourpi * r2 * e.ds);
+    e.thin = 1.0 / (fourpi * r2);
     geo[georow_index(m, a1, a2)] = e;
+    if (m <= kKapMax) {
+      const double2 k = kappa_dd(binom, m, a1, a2);
+      kap[georow_index(m, a1, a2)] = fma(k.x, e.ds, k.y * e.ds);
+      kappa[georow_index(m, a1, a2)] = k.x;
+    }
   }
 }
 
-cudaError_t launch_geometry(GeoEntry* geo, GeoRow* georow, int mmax, cudaStream_t s) {
+// k = min(mmax, kKapMax): binom is scratch of (k + 1)(k + 2)/2 double2, kap holds
+// georow_count(k) values of kappa ds and then as many of kappa
+cudaError_t launch_geometry(GeoEntry* geo, GeoRow* georow, double* kap, double2* binom, int mmax,
+                            cudaStream_t s) {
   if (mmax < 1) return cudaSuccess;
-  k_geometry_rows<<<mmax, 256, 0, s>>>(georow, mmax);
+  k_binomials<<<std::min(mmax, kKapMax) + 1, 64, 0, s>>>(binom, std::min(mmax, kKapMax));
+  count_launch();
+  k_geometry_rows<<<mmax, 256, 0, s>>>(georow, kap, kap + georow_count(std::min(mmax, kKapMax)), binom,
+                                       mmax);
   count_launch();
   k_geometry<<<mmax, 256, 0, s>>>(geo, mmax);
   count_launch();
@@ -518,10 +592,50 @@ __global__ void k_interior_tables(const int* __restrict__ ent_r2, const int* __r
     itab[off[e] + b] = 0;
 }
 
+// Cells of layer m of a whole face as signed offsets (t1, t2), two bytes each, in the
+// order that the in-place update of rates.cu needs, last first: quadrant positions (a1,
+// a2) by descending rows a1 and descending a2 (row a1 holds a2 = 0..min(H, isqrt(r2 - m^2 -
+// a1^2))), the distinct sign images of a position together.
+__global__ void k_face_tables(const int* __restrict__ ent_r2, const int* __restrict__ ent_m,
+                              const int4* __restrict__ lay, unsigned char* __restrict__ ftab,
+                              int nent) {
+  const int e = blockIdx.x;
+  if (e >= nent || lay[e].y == 0) return;
+  const int m = ent_m[e];
+  const int rem = ent_r2[e] - m * m;
+  const int H = min(isqrt_dev(rem), m);
+  char2* out = reinterpret_cast<char2*>(ftab + lay[e].x);
+  __shared__ int at[kFaceHcap + 1];  // first entry of row a1
+  if (threadIdx.x == 0) {
+    int run = 0;
+    for (int a1 = H; a1 >= 0; --a1) {
+      at[a1] = run;
+      run += (a1 ? 2 : 1) * (2 * min(H, isqrt_dev(rem - a1 * a1)) + 1);
+    }
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < (H + 1) * (H + 1); t += blockDim.x) {
+    const int a1 = t / (H + 1), a2 = t - a1 * (H + 1);
+    const int len = min(H, isqrt_dev(rem - a1 * a1));
+    if (a2 > len) continue;
+    const int n1 = a1 ? 2 : 1, n2 = a2 ? 2 : 1;
+    // (the cells are taken from the table's end)
+    char2* o = out + lay[e].z - 1 - (at[a1] + (len - a2) * 2 * n1);
+    for (int k = 0; k < n1 * n2; ++k)
+      o[-k] = make_char2((signed char)(k % n1 ? -a1 : a1), (signed char)(k / n1 ? -a2 : a2));
+  }
+  for (int t = threadIdx.x; t < lay[e].y / 2 - lay[e].z; t += blockDim.x)  // the padding
+    out[lay[e].z + t] = make_char2(0, 0);
+}
+
 void free_row_tables(Grid& g) {
   dev_free(g.rtab); dev_free(g.rtab_off); dev_free(g.rtab_first); dev_free(g.rtab_hcap);
-  dev_free(g.rtab_slot); dev_free(g.itab); dev_free(g.itab_off);
+  dev_free(g.rtab_slot); dev_free(g.rtab_lay); dev_free(g.ftab); dev_free(g.ftab_lay);
+  dev_free(g.itab); dev_free(g.itab_off);
   g.rtab = nullptr; g.rtab_off = g.rtab_first = g.rtab_hcap = g.rtab_slot = nullptr;
+  g.rtab_lay = nullptr;
+  g.ftab = nullptr; g.ftab_lay = nullptr;
+  g.ftab_bytes = 0;
   g.itab = nullptr; g.itab_off = nullptr;
   g.itab_bytes = 0;
   g.rtab_max_r2 = -1;
@@ -545,8 +659,9 @@ rt_status ensure_row_tables(Grid& g) {
     g.rtab_mcap = mcap;
     return RT_OK;
   }
+  std::vector<int4> lay, flay;
   std::vector<int> ent_r2, ent_m, off, ioff, first(r2s.size()), hcap(r2s.size());
-  int64_t cur = 0, icur = 0;
+  int64_t cur = 0, icur = 0, fcur = 0;
   for (size_t i = 0; i < r2s.size(); ++i) {
     const int v = r2s[i];
     const int L = std::min(isqrt_host(v), mcap);
@@ -566,6 +681,8 @@ rt_status ensure_row_tables(Grid& g) {
       ent_m.push_back(m);
       off.push_back((int)cur);
       ioff.push_back((int)icur);
+      lay.push_back(make_int4((int)cur, (int)((4 * (int64_t)(H + 2) + total + 15) & ~(int64_t)15),
+                              (int)total, H));
       cur += (4 * (int64_t)(H + 2) + total + 15) & ~(int64_t)15;
       icur += (4 * (int64_t)(LA + 1) + itotal + 15) & ~(int64_t)15;
       if (cur > (int64_t)1 << 30 || H > 254) {  // keep offsets in int, rows in bytes
@@ -575,6 +692,18 @@ rt_status ensure_row_tables(Grid& g) {
       }
     }
     hcap[i] = hc;
+    for (int m = 1; m <= L; ++m) {  // face tables of the narrow limits
+      if (hc > kFaceHcap) {
+        flay.push_back(make_int4(0, 0, 0, 0));
+        continue;
+      }
+      const int4 q = lay[first[i] + m - 1];
+      // four images of every position, less those that coincide on the two axes
+      const int n = 4 * q.z - 4 * (q.w + 1) + 1;
+      const int bytes = (2 * n + 15) & ~15;
+      flay.push_back(make_int4((int)fcur, bytes, n, q.w));
+      fcur += bytes;
+    }
   }
   off.push_back((int)cur);
   ioff.push_back((int)icur);
@@ -598,6 +727,12 @@ rt_status ensure_row_tables(Grid& g) {
   CK(dev_malloc(&g.rtab_first, first.size() * sizeof(int)));
   CK(dev_malloc(&g.rtab_hcap, hcap.size() * sizeof(int)));
   CK(dev_malloc(&g.rtab_slot, slot.size() * sizeof(int)));
+  CK(dev_malloc(&g.rtab_lay, std::max<size_t>(lay.size(), 1) * sizeof(int4)));
+  CK(cudaMemcpyAsync(g.rtab_lay, lay.data(), lay.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
+  CK(dev_malloc(&g.ftab, std::max<int64_t>(fcur, 16)));
+  CK(dev_malloc(&g.ftab_lay, std::max<size_t>(flay.size(), 1) * sizeof(int4)));
+  CK(cudaMemcpyAsync(g.ftab_lay, flay.data(), flay.size() * sizeof(int4), cudaMemcpyHostToDevice,
+                     s));
   CK(dev_malloc(&g.itab, std::max<int64_t>(icur, 16)));
   CK(dev_malloc(&g.itab_off, ioff.size() * sizeof(int)));
   CK(cudaMemcpyAsync(g.itab_off, ioff.data(), ioff.size() * sizeof(int), cudaMemcpyHostToDevice, s));
@@ -617,6 +752,11 @@ rt_status ensure_row_tables(Grid& g) {
     k_interior_tables<<<nent, 64, 0, s>>>(d_r2, d_m, g.itab_off, g.itab, nent);
     count_launch();
     CK(cudaGetLastError());
+    if (fcur > 0) {
+      k_face_tables<<<nent, 64, 0, s>>>(d_r2, d_m, g.ftab_lay, g.ftab, nent);
+      count_launch();
+      CK(cudaGetLastError());
+    }
   }
   CK(cudaStreamSynchronize(s));  // host vectors go out of scope
   dev_free(d_r2);
@@ -624,6 +764,7 @@ rt_status ensure_row_tables(Grid& g) {
   g.rtab_max_r2 = maxv;
   g.rtab_bytes = cur;
   g.itab_bytes = icur;
+  g.ftab_bytes = fcur;
   g.rtab_r2s = r2s;
   g.rtab_mcap = mcap;
   return RT_OK;

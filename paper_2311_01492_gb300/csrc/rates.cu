@@ -1,0 +1,647 @@
+// Batched trace of the photo-ionisation rates with the geometric weights
+// (RT_SCHED_BATCHED and its early exit; arXiv 2311.01492, Sec. 3.1-3.3).
+//
+// The work items, their order and the geometry are those of trace.cu: a face of a
+// source is a square pyramid whose layer m depends only on layer m - 1, split into
+// four quadrants.  An item is traced in two parts.
+//
+// While a layer has cells with tau_out below the tables' bound 2^E1, the recurrence
+// of trace.cu is evaluated as written there, so that every rate has the bits it has
+// in the other schedules.  Once every cell of a layer is beyond the bound, every
+// later tau_in (a convex combination plus non-negative increments) is too, and every
+// later rate is exactly 0: the early exit stops there, the full schedule goes on and
+// forms the remaining column densities in the scaled form below.
+//
+// Scaled form.  The geometric weights of a cell at transverse offsets (a1, a2) of
+// layer m are (1 - a1/m | a1/m) times (1 - a2/m | a2/m); with kappa_m(a1, a2) =
+// C(m, a1) C(m, a2) (binomial coefficients) and S = kappa tau_out they all become
+// one, by Pascal's rule C(m, a) (1 - a/m) = C(m-1, a), C(m, a) a/m = C(m-1, a-1):
+//
+//   v = kappa tau_in  = S(a1,a2) + S(a1-1,a2) + S(a1,a2-1) + S(a1-1,a2-1)
+//   S = kappa tau_out = fma(dtau, kappa ds, v)
+//
+// (S of layer m - 1 on the right of v; slots outside that layer are zero).  A cell
+// costs three additions and one fused multiply-add instead of five multiply-adds,
+// reads 8 bytes of geometry (kappa ds) instead of 40, and no weight is rounded.
+//
+// What binds: GB300 issues one FP64 warp instruction per 68-76 scheduler cycles,
+// but integer instructions at full rate beside it (measured: DFMA alone 76.1
+// cycles, DFMA with 64 integer instructions 78.3).  Two of the three additions
+// therefore run on the integer units, where they also round less: one bracket and
+// the final sum are formed as 64-bit integers with nine guard bits and rounded to
+// nearest once (<= 0.504 ulp of the sum).
+#include <algorithm>
+#include <cmath>
+#include <type_traits>
+
+#include "asora_internal.cuh"
+#include "device_util.cuh"
+#include "scaled_sum.cuh"
+
+namespace asora {
+
+// v of a cell from its four slots of the layer before: one addition on the FP64 unit,
+// two on the integer units.
+__device__ __forceinline__ double bracket_sum(double c1, double c2, double c3, double c4) {
+  return round_sum(c1 + c2, pair_sum(c3, c4));
+}
+
+// ------------------------------------------------------------ shared memory
+// Layer buffer: slot of (a1, a2), a1, a2 = -1..h, at (a1+1) W + a2+1, W = h+2 (row
+// and column -1 stay zero).  One buffer per warp (updated in place), two per CTA;
+// then `slots` row-table slots (device_util.cuh).
+__host__ __device__ inline size_t rates_buf_bytes(int h) {
+  return ((size_t)(h + 2) * (h + 2) * sizeof(double) + 15) & ~(size_t)15;
+}
+// Whole faces (mode 4): slot of the signed offsets (t1, t2) at (t1+h+1) W + t2+h+1, W =
+// 2h+3, slot 0 always zero; then two slots for the face tables (k_face_tables).
+__host__ __device__ inline size_t face_layer_bytes(int h) {
+  return ((size_t)(2 * h + 3) * (2 * h + 3) * sizeof(double) + 15) & ~(size_t)15;
+}
+__host__ __device__ inline int face_slot_bytes(int h) {
+  return (2 * (2 * h + 1) * (2 * h + 1) + 15) & ~15;
+}
+__host__ __device__ inline size_t rates_warp_bytes(int h, int mode) {
+  return mode == 4 ? face_layer_bytes(h) + 2 * (size_t)face_slot_bytes(h)
+                   : mode * rates_buf_bytes(h) + 2 * (size_t)row_slot_bytes(h);
+}
+static size_t rates_cta_bytes(int h, int slots) {
+  return 2 * rates_buf_bytes(h) + (size_t)slots * row_slot_bytes(h);
+}
+
+// Row-table slots of a CTA: the current layer's and the next's, or one (the next
+// layer's table then waits for the end of the layer) where two do not fit.
+static int cta_slots(int h) { return rates_cta_bytes(h, 2) <= 227 * 1024 ? 2 : 1; }
+
+size_t rates_smem_bytes(int hcap, int mode) {
+  return mode <= 4 ? rates_warp_bytes(hcap, mode) : rates_cta_bytes(hcap, cta_slots(hcap));
+}
+
+// ----------------------------------------------------------------- quadrants
+// One quadrant of a face as a lane sees it: the geometry of trace_face_item
+// (trace.cu) and its source's constants.
+struct Quad {
+  int N, R2, d, sg, q1, q2, lim1, lim2, Lmax;
+  int c1, c2, cd;          // source coordinates along t1, t2 and the face's axis
+  int md, st1;             // strides of the layer axis and (signed) of a1
+  int w1, w2, C1, C2;      // from a1 = w1 (a2 = w2) on, the offset is corrected by C1 (C2)
+  int org;                 // offset of (c1, c2) within a layer
+  int64_t off;             // first cell of the box
+  double half_dts, nd_thick, nd_thin;
+  const double* fld;       // dtau, rotated for the z faces: the stride of a2 is 1
+};
+
+__device__ __forceinline__ Quad quad_setup(const TraceArgs& a, const int item, const bool first,
+                                           unsigned& nrate) {
+  Quad Q;
+  const int s = item >> 5, f = (item >> 2) & 7, quad = item & 3;
+  const SrcDev S = a.src[s];
+  const BoxDev B = a.boxes[S.box];
+  const double nd = a.ndot[s];
+  Q.N = B.n;
+  Q.R2 = a.r2lim[s];
+  Q.d = f >> 1;
+  Q.sg = (f & 1) ? -1 : 1;
+  Q.q1 = (quad & 1) ? -1 : 1;
+  Q.q2 = (quad & 2) ? -1 : 1;
+  Q.lim1 = Q.q1 > 0 ? B.whi : -B.wlo;
+  Q.lim2 = Q.q2 > 0 ? B.whi : -B.wlo;
+  Q.Lmax = min(Q.sg > 0 ? B.whi : -B.wlo, isqrt_i(Q.R2));
+  Q.off = B.off;
+  const int64_t scell = B.off + ((int64_t)S.i * Q.N + S.j) * Q.N + S.k;
+  Q.half_dts = 0.5 * a.dtau[scell];
+  Q.nd_thick = nd * B.inv_cell3;
+  Q.nd_thin = nd * B.thin_fac;
+  if (f == 4 && quad == 0 && first) {  // the source cell (q = 0), once per source
+    double dG;
+    if (bits_of(Q.half_dts) <= bits_of(a.tau_lim))
+      dG = nd * (tab_eval(a.tab.h, a.tab, 0.0) * (0.5 * B.thin_fac));
+    else
+      dG = nd * ((tab_eval(a.tab.g, a.tab, 0.0) - tab_eval(a.tab.g, a.tab, Q.half_dts)) *
+                 B.inv_cell3);
+    ++nrate;
+    const bool thin = bits_of(Q.half_dts) <= bits_of(a.tau_lim);
+    if (dG != 0.0) atomicAdd(&(thin ? a.gamma : a.thick)[scell], dG);
+  }
+  const int NN = Q.N * Q.N;
+  Q.c1 = Q.d == 0 ? S.j : S.i;
+  Q.c2 = Q.d == 2 ? S.j : S.k;
+  Q.cd = Q.d == 0 ? S.i : (Q.d == 1 ? S.j : S.k);
+  const int m1 = Q.d == 1 ? NN : Q.N;
+  Q.md = Q.d == 1 ? Q.N : NN;
+  Q.fld = (Q.d == 2 ? a.dtauT : a.dtau) + B.off;
+  Q.st1 = Q.q1 * m1;
+  Q.w1 = Q.q1 > 0 ? Q.N - Q.c1 : Q.c1 + 1;
+  Q.w2 = Q.q2 > 0 ? Q.N - Q.c2 : Q.c2 + 1;
+  Q.C1 = -Q.q1 * Q.N * m1;
+  Q.C2 = -Q.q2 * Q.N;
+  Q.org = Q.c1 * m1 + Q.c2;
+  return Q;
+}
+
+// First layer entry (rtab_lay) of the item's R^2 limit, or -1 if a window of half-width
+// lim clips a layer (or there are no tables).
+__device__ __forceinline__ int first_layer_entry(const TraceArgs& a, const int R2, const int lim) {
+  if (R2 > a.rtab_max_r2) return -1;
+  const int sl = a.rtab_slot[R2];
+  return sl >= 0 && a.rtab_hcap[sl] <= lim ? a.rtab_first[sl] : -1;
+}
+
+// One cell in flight: transverse offsets along the item's signs (quadrants: >= 0) or
+// signed (faces).
+struct CellIn {
+  int t1, t2, gidx;
+  double dtp, kds;
+};
+
+__device__ __forceinline__ void fetch_cell(const Quad& Q, CellIn& c, const int t, const int base,
+                                           const int* __restrict__ rowpre,
+                                           const unsigned char* __restrict__ rowof) {
+  c.t1 = rowof[t];
+  c.t2 = t - rowpre[c.t1];
+  c.gidx = base + c.t1 * Q.st1 + Q.q2 * c.t2 + (c.t1 >= Q.w1 ? Q.C1 : 0) + (c.t2 >= Q.w2 ? Q.C2 : 0);
+  c.dtp = __ldg(&Q.fld[c.gidx]);
+}
+
+// The same from a face table; a face wraps on either side.
+__device__ __forceinline__ void fetch_face_cell(const Quad& Q, CellIn& c, const int t,
+                                                const int base, const char2* __restrict__ cells) {
+  const char2 v = cells[t];
+  c.t1 = v.x;
+  c.t2 = v.y;
+  const int x1 = Q.c1 + c.t1, x2 = Q.c2 + c.t2;
+  c.gidx = base + c.t1 * Q.st1 + c.t2 + (x1 < 0 ? -Q.C1 : x1 >= Q.N ? Q.C1 : 0) +
+           (x2 < 0 ? -Q.C2 : x2 >= Q.N ? Q.C2 : 0);
+  c.dtp = __ldg(&Q.fld[c.gidx]);
+}
+
+// Weights and path length of a cell.
+struct Weights {
+  double2 w12, w34;
+  double ds;
+};
+__device__ __forceinline__ Weights load_weights(const GeoRow* __restrict__ gr) {
+  return {__ldg(reinterpret_cast<const double2*>(gr)),
+          __ldg(reinterpret_cast<const double2*>(gr) + 1), __ldg(&gr->ds)};
+}
+
+// tau_in of a cell from the interpolants at slot s and up to d1 and d2 before it
+// (trace.cu; the slots that a zero weight reads hold a finite value).
+__device__ __forceinline__ double interp(const TraceArgs& a, const Weights& w, const double* s,
+                                         const int d1, const int d2) {
+  return fma(w.w34.y, s[-d1 - d2],
+             fma(w.w34.x, s[-d2], fma(w.w12.y, s[-d1], fma(w.w12.x, s[0], a.neg_zero))));
+}
+
+// The rate of a cell of layer m >= 1 whose tau_in is within the tables (Eq. sugg; thin
+// limit Eq. gammalocal).  The thick terms are summed without their factor 1/n_HI,
+// which is the cell's own and is applied once to the sum (k_add_thick): one product
+// and one gather less per rate.  dtau ds is formed only where dtau is not above
+// tau_lim by its high word (ds >= 1).  FACE: a face's cells are its own but for the
+// ties; a quadrant's also leave out the lines that it shares with the one before it.
+template <bool FACE>
+__device__ __forceinline__ void deposit_rate(const TraceArgs& a, const Quad& Q, const int m,
+                                             const CellIn& c, const GeoRow* __restrict__ gr,
+                                             const double ds, const double tin, const double tout,
+                                             unsigned& nrate) {
+  const int a1 = FACE ? abs(c.t1) : c.t1, a2 = FACE ? abs(c.t2) : c.t2;
+  const bool own = ((Q.d == 2) || (Q.d == 1 ? a2 < m : (a1 < m && a2 < m))) &&
+                   (FACE || ((a1 > 0 || Q.q1 > 0) && (a2 > 0 || Q.q2 > 0)));
+  if (!own) return;
+  const double2 gv = __ldg(reinterpret_cast<const double2*>(gr) + 3);  // invv, thin
+  int64_t cell = Q.off + c.gidx;
+  if (Q.d == 2) {  // gathered from the rotated copy
+    const int x1 = wrapc(Q.c1 + Q.q1 * c.t1, Q.N), x2 = wrapc(Q.c2 + Q.q2 * c.t2, Q.N);
+    cell = Q.off + (x1 * Q.N + x2) * Q.N + wrapc(Q.cd + Q.sg * m, Q.N);
+  }
+  bool thin = __double2hiint(c.dtp) <= __double2hiint(a.tau_lim);
+  if (thin) thin = bits_of(c.dtp * ds) <= bits_of(a.tau_lim);
+  double* out;
+  double dG;
+  if (thin) {
+    out = a.gamma;
+    dG = Q.nd_thin * (tab_eval(a.tab.h, a.tab, tin) * gv.y);
+  } else {
+    out = a.thick;
+    dG = Q.nd_thick * ((tab_eval(a.tab.g, a.tab, tin) - tab_eval(a.tab.g, a.tab, tout)) * gv.x);
+  }
+  ++nrate;
+  if (dG != 0.0) atomicAdd(&out[cell], dG);
+}
+
+// Doubles of the part of a layer buffer that an item can read before it writes it
+// (the rim of each layer), from the buffer's start.
+__device__ __forceinline__ int zero_count(int R2, int h) {
+  return (min(h, isqrt_i(R2 >> 1)) + 2) * (h + 2);
+}
+
+// tau_out -> S for the cells of layer m (and whatever else lies in its square).
+template <int GS>
+__device__ __forceinline__ void scale_layer(const TraceArgs& a, double* buf, const int W,
+                                            const int m, const int h, const int gt) {
+  const int H = min(m, h) + 1;
+  const double* __restrict__ k = a.kappa + georow_index(m, 0, 0);
+  for (int t = gt; t < H * H; t += GS) {
+    const int a1 = t / H, a2 = t - a1 * H;
+    buf[(a1 + 1) * W + a2 + 1] *= __ldg(&k[a1 * (m + 1) + a2]);
+  }
+}
+
+// The same for a whole face.
+__device__ __forceinline__ void scale_face(const TraceArgs& a, double* buf, const int W, const int m,
+                                           const int h, const int lane) {
+  const int H = min(m, h), S = 2 * H + 1;
+  const double* __restrict__ k = a.kappa + georow_index(m, 0, 0);
+  for (int t = lane; t < S * S; t += 32) {
+    const int t1 = t / S - H, t2 = t % S - H;
+    buf[(t1 + h + 1) * W + t2 + h + 1] *= __ldg(&k[abs(t1) * (m + 1) + abs(t2)]);
+  }
+}
+
+// MODE 1, 2: as many quadrants of one face (from `item` on) by one warp, 32 / MODE
+// lanes each with a layer buffer of its own: the quadrants have the same cells, so they
+// share the row tables, the geometry loads and the work per layer.  A buffer is updated
+// in place, in descending flat order: the slots a cell reads have flat indices not
+// above its own, so none is rewritten before it is read.
+// MODE 4: a whole face by one warp, for small layers, where the axis lines that two
+// quadrants share are a large part (1.25 cells per cell of the ball at R = 15, 1.47 at
+// 8).  The cells of a layer come from a table (k_face_tables) in descending order of
+// their quadrant position, the images of a position together: the same argument holds.
+// The indices and dtau of the next cells (of the next layer at a layer's
+// end) are loaded before a step is computed; a step of the scaled part takes two sets
+// of 32 cells, whose chains overlap.
+template <int MODE, bool EXIT>
+__device__ __forceinline__ void rates_item_warp(const TraceArgs& a, const int item, const int lane,
+                                                unsigned char* __restrict__ sm, const int h,
+                                                unsigned& nrate) {
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr bool FACE = MODE == 4;
+  constexpr int K = FACE ? 1 : MODE;
+  constexpr int P = 32 / K;  // lanes, and cells of a set, per quadrant (or face)
+  const int W = FACE ? 2 * h + 3 : h + 2;
+  const int TS = FACE ? face_slot_bytes(h) : row_slot_bytes(h);
+  const int lq = lane % P;
+  const Quad Q = quad_setup(a, item + lane / P, lane == 0, nrate);
+  double* buf = reinterpret_cast<double*>(sm + (FACE ? 0 : (lane / P) * rates_buf_bytes(h)));
+  unsigned char* tab = sm + (FACE ? face_layer_bytes(h) : K * rates_buf_bytes(h));
+  double* const org = FACE ? buf + (h + 1) * (W + 1) : buf + W + 1;  // slot of (0, 0)
+  if (FACE) {
+    const int hz = min(h, isqrt_i(Q.R2 >> 1));
+    for (int t = (h - hz) * W + lane; t < (h + hz + 3) * W; t += 32) buf[t] = 0.0;
+    if (lane == 0) buf[0] = 0.0;
+  } else {
+    for (int t = lq, n = zero_count(Q.R2, h); t < n; t += P) buf[t] = 0.0;
+  }
+  if (Q.Lmax < 1) return;
+  // the row tables serve all K quadrants: those of a window wider by one cell on one
+  // side leave cells out (in_window below); the face tables know no window
+  const int lim1 = K > 1 ? max(Q.lim1, __shfl_xor_sync(FULL, Q.lim1, P)) : Q.lim1;
+  const int lmin1 = K > 1 ? min(Q.lim1, __shfl_xor_sync(FULL, Q.lim1, P)) : Q.lim1;
+  const int ent = first_layer_entry(a, Q.R2, FACE ? h : min(lmin1, Q.lim2));
+  const int4* __restrict__ lays = FACE ? a.ftab_lay : a.rtab_lay;
+  const unsigned char* __restrict__ blobs = FACE ? a.ftab : a.rtab;
+
+  // fetch side: the layer whose cells are being loaded
+  int m = 0, sq = 0, kofs = -1, base = 0, T0 = -1;
+  // layers m + 1 and m + 2: blob offset, bytes, cells, half-width
+  int4 lay = make_int4(0, 0, 0, 0), lay2 = lay;
+  const int* rowpre = nullptr;
+  const unsigned char* rowof = nullptr;
+  const char2* cells = nullptr;
+  bool bad = FACE && ent < 0;
+  auto stage = [&]() {  // table of layer m + 1
+    unsigned char* dst = tab + ((m + 1) & 1) * TS;
+    if (FACE || ent >= 0) {
+      if (lay.y > TS) bad = true;
+      else stage_rows<32>(blobs + lay.x, lay.y, dst, lane);
+    } else {
+      while (sq * sq > Q.R2 - (m + 1) * (m + 1)) --sq;
+      const int H = min(m + 1, sq);
+      if (H > h) {
+        bad = true;
+      } else {
+        const int nr = min(H, lim1) + 1;
+        int* pre = reinterpret_cast<int*>(dst);
+        quad_rows_warp(Q.R2 - (m + 1) * (m + 1), H, nr, Q.lim2, pre,
+                       reinterpret_cast<unsigned char*>(pre + nr + 1), lane);
+        lay.w = nr - 1;
+      }
+    }
+  };
+  auto next_layer = [&]() {  // makes m + 1 the fetched layer (its table has been staged)
+    cp_async_wait_all();
+    __syncwarp();
+    T0 = -1;
+    if (bad || m >= Q.Lmax || m >= a.kap_mmax) {
+      if ((bad || m < Q.Lmax) && lane == 0) atomicOr(a.err, bad ? ERR_LAYER_CAP : ERR_GEO);
+      return;
+    }
+    ++m;
+    kofs += m * m;
+    if (FACE) {
+      cells = reinterpret_cast<const char2*>(tab + (m & 1) * TS);
+      T0 = lay.z - 1;
+    } else {
+      rowpre = reinterpret_cast<const int*>(tab + (m & 1) * TS);
+      rowof = reinterpret_cast<const unsigned char*>(rowpre + lay.w + 2);
+      T0 = (ent >= 0 ? lay.z : rowpre[lay.w + 1]) - 1;
+    }
+    base = wrapc(Q.cd + Q.sg * m, Q.N) * Q.md + Q.org;
+    if (m < Q.Lmax) {
+      if (FACE || ent >= 0) {
+        lay = lay2;
+        if (m + 1 < Q.Lmax) lay2 = __ldg(&lays[ent + m + 1]);
+      }
+      stage();
+    }
+  };
+  auto in_window = [&](const CellIn& c) {
+    return (K == 1 && !FACE) || (c.t1 <= Q.lim1 && c.t2 <= Q.lim2);
+  };
+  auto fetch = [&](CellIn& c, int t) {  // the cell and its offset in the geometry rows
+    if (FACE) fetch_face_cell(Q, c, t, base, cells);
+    else fetch_cell(Q, c, t, base, rowpre, rowof);
+    return kofs + (FACE ? abs(c.t1) : c.t1) * (m + 1) + (FACE ? abs(c.t2) : c.t2);
+  };
+  // slots one step towards the source along t1 and t2 (faces: the slot itself on an axis)
+  auto d1_of = [&](const CellIn& c) { return FACE ? sgn_i(c.t1) * W : W; };
+  auto d2_of = [&](const CellIn& c) { return FACE ? sgn_i(c.t2) : 1; };
+
+  sq = isqrt_i(Q.R2 - 1);
+  if (ent >= 0) {
+    lay = __ldg(&lays[ent]);
+    if (Q.Lmax > 1) lay2 = __ldg(&lays[ent + 1]);
+  }
+  if (!bad) stage();
+  next_layer();
+  if (T0 < 0) return;
+  // ---- cells with rates
+  bool opaque = true;  // every cell of this lane in the layer has tau_out beyond the bound
+  CellIn nc;
+  Weights nw;
+  const GeoRow* ng;
+  auto prefetch_rated = [&]() {
+    ng = a.georow + fetch(nc, max(T0 - lq, 0));
+    nw = load_weights(ng);
+  };
+  prefetch_rated();
+  // A layer's last step ends with the test whether all of it is opaque (2^E1 (1 + 2^-40);
+  // the margin covers the rounding of later layers).
+  auto step = [&](auto first) {
+    constexpr bool FIRST = decltype(first)::value;
+    const CellIn c = nc;
+    const Weights w = nw;
+    const GeoRow* gr = ng;
+    const int mc = m, Tc = T0;
+    const bool last = Tc < P;
+    T0 -= P;
+    if (last) next_layer();
+    if (T0 >= 0) prefetch_rated();
+    double* sc = org + c.t1 * W + c.t2;
+    double tin;
+    if constexpr (FIRST) tin = Q.half_dts * w.ds;  // source centre to the layer's entry plane
+    else tin = interp(a, w, sc, d1_of(c), d2_of(c));
+    const double tout = fma(c.dtp, w.ds, tin);
+    __syncwarp();  // all reads before any write
+    if (Tc - lq >= 0 && in_window(c)) {
+      *sc = tout;
+      opaque = opaque && bits_of(tout) >= a.exit_bits;
+      if (bits_of(tin) < a.tab.tau_max_bits)
+        deposit_rate<FACE>(a, Q, mc, c, gr, w.ds, tin, tout, nrate);
+    }
+    __syncwarp();
+    if (!last) return false;
+    const bool all = __all_sync(FULL, opaque);
+    opaque = true;
+    return all;
+  };
+  bool done = step(std::true_type());
+  while (T0 >= 0 && !done) done = step(std::false_type());
+  if (EXIT || T0 < 0) {
+    cp_async_wait_all();  // (a copy may be in flight)
+    return;
+  }
+  // ---- no rates any more: the column densities in scaled form
+  if (FACE) scale_face(a, buf, W, m - 1, h, lane);
+  else scale_layer<P>(a, buf, W, m - 1, h, lq);
+  __syncwarp();
+  CellIn ne;
+  auto prefetch = [&]() {
+    nc.kds = __ldg(&a.kap[fetch(nc, max(T0 - lq, 0))]);
+    if (T0 >= P) ne.kds = __ldg(&a.kap[fetch(ne, max(T0 - P - lq, 0))]);
+  };
+  auto column = [&](const CellIn& c, const double* s) {  // S of the cell at slot s
+    const int d1 = d1_of(c), d2 = d2_of(c);
+    const bool z1 = FACE && c.t1 == 0, z2 = FACE && c.t2 == 0;  // nothing beyond an axis
+    const double v = bracket_sum(s[0], z1 ? buf[0] : s[-d1], z2 ? buf[0] : s[-d2],
+                                 z1 || z2 ? buf[0] : s[-d1 - d2]);
+    return fma(c.dtp, c.kds, v);
+  };
+  prefetch();
+  while (T0 >= 0) {
+    const CellIn c = nc, e = ne;
+    const int Tc = T0;
+    T0 -= 2 * P;
+    if (T0 < 0) next_layer();
+    if (T0 >= 0) prefetch();
+    double* sc = org + c.t1 * W + c.t2;
+    const bool in_c = Tc - lq >= 0 && in_window(c);
+    if (Tc >= P) {  // (one block, so that the two chains interleave)
+      double* se = org + e.t1 * W + e.t2;
+      const double v = column(c, sc);
+      const double y = column(e, se);
+      __syncwarp();  // all reads before any write
+      if (in_c) *sc = v;
+      if (Tc - P - lq >= 0 && in_window(e)) *se = y;
+    } else {
+      const double v = column(c, sc);
+      __syncwarp();
+      if (in_c) *sc = v;
+    }
+    __syncwarp();
+  }
+}
+
+// One quadrant item by a CTA of GS threads (large sources): two layer buffers and a
+// barrier per layer.
+template <int GS, bool EXIT>
+__device__ __forceinline__ void rates_item_cta(const TraceArgs& a, const int item, const int gt,
+                                               unsigned char* __restrict__ sm, const int h,
+                                               const int slots, unsigned& nrate) {
+  const int W = h + 2;
+  const int TS = row_slot_bytes(h);
+  double* cur = reinterpret_cast<double*>(sm);
+  double* prev = reinterpret_cast<double*>(sm + rates_buf_bytes(h));
+  unsigned char* tab = sm + 2 * rates_buf_bytes(h);
+  const int wid = gt >> 5, lane = gt & 31;
+  const Quad Q = quad_setup(a, item, gt == 0, nrate);
+  for (int t = gt, n = zero_count(Q.R2, h); t < n; t += GS) cur[t] = prev[t] = 0.0;
+  const int ent = first_layer_entry(a, Q.R2, min(Q.lim1, Q.lim2));
+  auto slot_of = [&](int m) { return tab + (slots == 2 ? (m & 1) * TS : 0); };
+  auto stage = [&](int m, int H) {  // row table of layer m (waited for separately)
+    if (ent >= 0) {
+      const int4 lay = __ldg(&a.rtab_lay[ent + m - 1]);
+      stage_rows<GS>(a.rtab + lay.x, lay.y, slot_of(m), gt);
+    } else if (wid == 0) {
+      const int nr = min(H, Q.lim1) + 1;
+      int* pre = reinterpret_cast<int*>(slot_of(m));
+      quad_rows_warp(Q.R2 - m * m, H, nr, Q.lim2, pre,
+                     reinterpret_cast<unsigned char*>(pre + nr + 1), lane);
+    }
+  };
+  if (Q.Lmax >= 1) {
+    const int H1 = min(1, isqrt_i(Q.R2 - 1));
+    if (H1 <= h) stage(1, H1);
+    cp_async_wait_all();
+  }
+  group_sync<GS>();
+  bool scaled = false;
+  for (int m = 1; m <= Q.Lmax; ++m) {
+    const int H = min(m, isqrt_i(Q.R2 - m * m));
+    if (H > h || m > a.kap_mmax) {
+      if (gt == 0) atomicOr(a.err, H > h ? ERR_LAYER_CAP : ERR_GEO);
+      break;
+    }
+    const int nrows = min(H, Q.lim1) + 1;
+    const int* rowpre = reinterpret_cast<const int*>(slot_of(m));
+    const unsigned char* rowof = reinterpret_cast<const unsigned char*>(rowpre + nrows + 1);
+    const int total = rowpre[nrows];
+    int Hn = 0;  // half-width of the next layer
+    if (m < Q.Lmax) {
+      Hn = min(m + 1, isqrt_i(Q.R2 - (m + 1) * (m + 1)));
+      if (slots == 2 && Hn <= h && ent >= 0) stage(m + 1, Hn);
+    }
+    const int base = wrapc(Q.cd + Q.sg * m, Q.N) * Q.md + Q.org;
+    const int gofs = (int)georow_index(m, 0, 0);
+    bool opaque = true;  // every cell of this thread has tau_out beyond the bound
+    CellIn c;
+    if (scaled) {
+      for (int t = gt; t < total; t += GS) {
+        fetch_cell(Q, c, t, base, rowpre, rowof);
+        const double kds = __ldg(&a.kap[gofs + c.t1 * (m + 1) + c.t2]);
+        const int o = (c.t1 + 1) * W + c.t2 + 1;
+        const double* s = prev + o;
+        cur[o] = fma(c.dtp, kds, bracket_sum(s[0], s[-W], s[-1], s[-W - 1]));
+      }
+    } else {
+      auto cells = [&](auto first) {
+        constexpr bool FIRST = decltype(first)::value;
+        for (int t = gt; t < total; t += GS) {
+          fetch_cell(Q, c, t, base, rowpre, rowof);
+          const GeoRow* gr = a.georow + gofs + c.t1 * (m + 1) + c.t2;
+          const int o = (c.t1 + 1) * W + c.t2 + 1;
+          const Weights w = load_weights(gr);
+          double tin;
+          if constexpr (FIRST) tin = Q.half_dts * w.ds;
+          else tin = interp(a, w, prev + o, W, 1);
+          const double tout = fma(c.dtp, w.ds, tin);
+          cur[o] = tout;
+          opaque = opaque && bits_of(tout) >= a.exit_bits;
+          if (bits_of(tin) < a.tab.tau_max_bits)
+            deposit_rate<false>(a, Q, m, c, gr, w.ds, tin, tout, nrate);
+        }
+      };
+      if (m == 1) cells(std::true_type());
+      else cells(std::false_type());
+    }
+    if (m < Q.Lmax && Hn <= h) {  // row table of the next layer
+      if (slots == 1) group_sync<GS>();  // this layer's is no longer read
+      if (slots == 1 || ent < 0) stage(m + 1, Hn);
+      cp_async_wait_all();
+    }
+    if (scaled) {
+      group_sync<GS>();
+    } else if (__syncthreads_and(opaque)) {  // as in rates_item_warp
+      if (EXIT) break;
+      scaled = true;
+      scale_layer<GS>(a, cur, W, m, h, gt);
+      group_sync<GS>();
+    }
+    double* tmp = prev;
+    prev = cur;
+    cur = tmp;
+  }
+}
+
+__device__ __forceinline__ void flush_rates(const TraceArgs& a, unsigned nrate) {
+  if (!a.rate_cells) return;
+  for (int o = 16; o > 0; o >>= 1) nrate += __shfl_down_sync(0xffffffffu, nrate, o);
+  if ((threadIdx.x & 31) == 0 && nrate) atomicAdd(a.rate_cells, (unsigned long long)nrate);
+}
+
+template <int BLOCK, bool EXIT>
+__global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) k_rates_cta(TraceArgs a, int slots) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int s_item;
+  if (a.skip && *a.skip) return;
+  unsigned nrate = 0;
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) s_item = a.item_begin + atomicAdd(a.queue, 1);
+    __syncthreads();
+    const int it = s_item;
+    if (it >= a.n_items) break;
+    rates_item_cta<BLOCK, EXIT>(a, a.items[it], threadIdx.x, smem_raw, a.hcap, slots, nrate);
+  }
+  flush_rates(a, nrate);
+}
+
+template <int MODE, bool EXIT>
+__global__ void __launch_bounds__(256, 2) k_rates_warp(TraceArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (a.skip && *a.skip) return;
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned char* my = smem_raw + (size_t)wid * rates_warp_bytes(a.hcap, MODE);
+  unsigned nrate = 0;
+  for (;;) {
+    int it = 0;
+    if (lane == 0) it = a.item_begin + atomicAdd(a.queue, 1);
+    it = __shfl_sync(0xffffffffu, it, 0);
+    if (it >= a.n_items) break;
+    rates_item_warp<MODE, EXIT>(a, a.items[it * MODE], lane, my, a.hcap, nrate);
+    __syncwarp();
+  }
+  flush_rates(a, nrate);
+}
+
+// mode: quadrants per warp (1, 2), 4: a whole face per warp, or threads of a CTA (128, 256)
+static const void* rates_kernel(int mode, bool exit) {
+#define ASORA_PICK(...) (exit ? (const void*)__VA_ARGS__, true> : (const void*)__VA_ARGS__, false>)
+  switch (mode) {
+    case 1: return ASORA_PICK(k_rates_warp<1);
+    case 2: return ASORA_PICK(k_rates_warp<2);
+    case 4: return ASORA_PICK(k_rates_warp<4);
+    case 128: return ASORA_PICK(k_rates_cta<128);
+    case 256: return ASORA_PICK(k_rates_cta<256);
+    default: return nullptr;
+  }
+#undef ASORA_PICK
+}
+
+cudaError_t launch_rates(Grid& g, const TraceArgs& a, int mode, int grid, size_t smem, int wpb) {
+  const void* fn = rates_kernel(mode, a.early_exit != 0);
+  if (!fn) return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  TraceArgs arg = a;
+  int slots = mode <= 4 ? 2 : cta_slots(a.hcap);
+  void* params[] = {&arg, &slots};
+  e = cudaLaunchKernel(fn, dim3(grid), dim3(mode <= 4 ? wpb * 32 : mode), params, smem, g.stream);
+  count_launch();
+  return e;
+}
+
+int rates_max_grid(int mode, size_t smem, int wpb, bool exit) {
+  int dev = 0, sms = 0, per = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const void* fn = rates_kernel(mode, exit);
+  if (!fn) return 0;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, mode <= 4 ? wpb * 32 : mode, smem);
+  if (e != cudaSuccess) return 0;
+  return per * sms;
+}
+
+}  // namespace asora

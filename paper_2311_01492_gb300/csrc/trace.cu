@@ -16,7 +16,9 @@
 // a CTA-wide barrier between shells, keeping the column densities of its
 // source in a private cube of global memory.
 //
-// k_trace_faces (RT_SCHED_BATCHED) is the GB300 schedule.  The interpolants of
+// k_trace_faces (RT_SCHED_BATCHED) is the GB300 schedule, here for a source's column
+// densities and for the rates with optical-depth-modulated weights (the rates with the
+// geometric weights, whose items are the same, are in rates.cu).  The interpolants of
 // a cell whose dominant axis is d lie in the plane one step closer to the
 // source along d (Eq. raga, entry plane), so the cells with dominant axis d
 // and sign +-1 -- a square pyramid ("face") -- form layers m = 1, 2, ... that
@@ -713,27 +715,21 @@ __global__ void __launch_bounds__(256, 3) k_trace_faces_whole_warp(TraceArgs a) 
 
 // Kernel variant for (block, warps per CTA, coldens): block 128/256 = CTA mode,
 // 32 = warp mode and 4 = whole-face warp mode with wpb warps per CTA (1..8).  Null
-// if not instantiated.
+// if not instantiated.  (The rates with the geometric weights are traced by rates.cu:
+// without od, the variant that writes column densities is the only one.)
 static const void* face_kernel(int block, int wpb, bool coldens, bool od) {
-#define ASORA_PICK(K) (od ? (coldens ? (const void*)K<true, true> : (const void*)K<false, true>) \
-                          : (coldens ? (const void*)K<true, false> : (const void*)K<false, false>))
+#define ASORA_PICK(...)                                                             \
+  (!od ? (const void*)__VA_ARGS__ true, false> : coldens ? (const void*)__VA_ARGS__ true, true> \
+                                                         : (const void*)__VA_ARGS__ false, true>)
   switch (block) {
     case 32:
       if (wpb < 1 || wpb > 8) return nullptr;
-      return ASORA_PICK(k_trace_faces_warp);
+      return ASORA_PICK(k_trace_faces_warp<);
     case 4:  // whole-face warp mode, wpb warps per CTA
       if (wpb < 1 || wpb > 8) return nullptr;
-      return ASORA_PICK(k_trace_faces_whole_warp);
-    case 128:
-      return od ? (coldens ? (const void*)k_trace_faces<128, true, true>
-                           : (const void*)k_trace_faces<128, false, true>)
-                : (coldens ? (const void*)k_trace_faces<128, true, false>
-                           : (const void*)k_trace_faces<128, false, false>);
-    case 256:
-      return od ? (coldens ? (const void*)k_trace_faces<256, true, true>
-                           : (const void*)k_trace_faces<256, false, true>)
-                : (coldens ? (const void*)k_trace_faces<256, true, false>
-                           : (const void*)k_trace_faces<256, false, false>);
+      return ASORA_PICK(k_trace_faces_whole_warp<);
+    case 128: return ASORA_PICK(k_trace_faces<128,);
+    case 256: return ASORA_PICK(k_trace_faces<256,);
     default: return nullptr;
   }
 #undef ASORA_PICK
