@@ -269,6 +269,12 @@ static int first_fitting(const Grid& g, const int* r2s, int ns, int hlim) {
   return lo;
 }
 
+// Threads of a CTA that has an SM to itself, for layers of half-width h.  One source, us
+// a pass with 128 / 256 / 512 threads (column densities; rates in an ionised box): R = 16
+// (h = 11) 50 / 50 / 52; 51 / 54 / 55; R = 24 (16) 70 / 66 / 68; 83 / 76 / 79; R = 40 (28)
+// 168 / 137 / 133; 223 / 176 / 169; R = 70 (49) 566 / 382 / 321; 881 / 537 / 454.
+static int few_items_block(int h) { return (h < 12 ? 128 : h < 24 ? 256 : 512) | kAhead; }
+
 // Launches of the batched rates: sources [cut[k], cut[k+1]) (LPT order) by CTAs of
 // mode[0] threads (k = 0) or by warps with one quadrant, two, or a whole face (k = 1..3).
 struct RatesPlan {
@@ -286,7 +292,9 @@ struct RatesPlan {
 // one before it (64^3, 1e3 sources of R = 5..50: one launch 0.52, three 0.87 ms), and
 // where one quadrant would take a warp longer than all work takes the GPU, CTAs trace
 // everything (64^3, 10 sources of R = 20: 0.048 against 0.057 ms; 128^3, 40 of R = 40:
-// 0.123 / 0.187), of 256 threads where not even every SM gets two.
+// 0.123 / 0.187).  With at most two items per SM they are the kAhead ones; with up to
+// four, CTAs of 256 pay for wide layers (200^3, 20 sources of R = 45: 0.146 / 0.177;
+// 128^3, 40 of R = 40, six items per SM: 0.156 / 0.128).
 static RatesPlan rates_plan(const Grid& g, const int* r2s, int ns) {
   RatesPlan p;
   p.mode[0] = g.block_big;
@@ -304,7 +312,9 @@ static RatesPlan rates_plan(const Grid& g, const int* r2s, int ns) {
   const double ball = std::min(4.18879 * r * r * r, (double)g.nmax * g.nmax * g.nmax);
   p.mode[0] = 128;
   if (ball * warps > 1.2 * 24 * (double)g.source_voxels) {
-    if (24 * ns <= 2 * sms && face_hcap(r2s[0], g.nmax) >= 24) p.mode[0] = 256;
+    const int h = face_hcap(r2s[0], g.nmax);
+    if (24 * ns <= 2 * sms) p.mode[0] = few_items_block(h);
+    else if (24 * ns <= 4 * sms && h >= 24) p.mode[0] = 256;
     p.cut[1] = p.cut[2] = p.cut[3] = ns;
     return p;
   }
@@ -352,10 +362,10 @@ static rt_status run_rates(Grid& g, const TraceArgs& a, const int* items, int ns
     }
     if (maxg <= 0) return fail(RT_ERR_CUDA, "rt_raytrace: no occupancy for a rate kernel");
     const int nitem = b.n_items - b.item_begin;
-    const int grid = std::max(1, std::min((nitem + wpb - 1) / wpb, maxg));
+    const int grid = mode[k] & kAhead ? nitem : std::max(1, std::min((nitem + wpb - 1) / wpb, maxg));
     TRY(launch_rates(g, b, mode[k], grid, smem * wpb, wpb));
     if (++g.stats.launches == 1) {
-      g.stats.block = k == 0 ? mode[k] : 32 * wpb;
+      g.stats.block = k == 0 ? mode[k] & ~kAhead : 32 * wpb;
       g.stats.grid = grid;
     }
   }
@@ -690,8 +700,8 @@ rt_status rt_raytrace(rt_grid_t h, double* d_gamma, int schedule) {
   if (st != RT_OK) return st;
   if (schedule == RT_SCHED_AUTO) schedule = g.auto_plain ? RT_SCHED_PLAIN : RT_SCHED_BATCHED;
   TRY(cudaEventRecord(g.ev[0], g.stream));
-  TRY(launch_precompute(g, schedule != RT_SCHED_PLAIN && takes_rates_kernels(g)));
-  TRY(cudaMemsetAsync(d_gamma, 0, g.ncell * sizeof(double), g.stream));
+  TRY(launch_precompute(g, schedule != RT_SCHED_PLAIN && takes_rates_kernels(g) ? PRE_THICK : PRE_INVN,
+                        d_gamma));
   TRY(cudaEventRecord(g.ev[1], g.stream));
   if (g.nsrc > 0) {
     if (schedule == RT_SCHED_PLAIN)
@@ -717,14 +727,33 @@ rt_status rt_raytrace_source_coldens(rt_grid_t h, int src, double* d_coldens, in
     return fail(RT_ERR_INVALID, "rt_raytrace_source_coldens: source index out of range");
   rt_status st = check_ready(g, "rt_raytrace_source_coldens");
   if (st != RT_OK) return st;
+  TRY(launch_precompute(g, PRE_DTAU, d_coldens));
+  const int hmax = face_hcap(g.max_r2, g.nmax);
+  if (schedule != RT_SCHED_PLAIN && takes_rates_kernels(g) && g.nmax <= 1290 &&
+      rates_smem_bytes(hmax, few_items_block(hmax)) <= 227 * 1024) {
+    // 24 CTAs, their source looked up on the device, with room for the widest one:
+    // nothing is asked back
+    TraceArgs a = base_args(g);
+    a.coldens = d_coldens;
+    a.one_src = g.src_of_input + src;
+    a.hcap = hmax;
+    const int block = few_items_block(hmax);
+    TRY(launch_rates(g, a, block, 24, rates_smem_bytes(hmax, block), 1));
+    TRY(launch_tau_to_coldens(g, d_coldens));
+    g.stats.launches = 1;
+    g.stats.block = block & ~kAhead;
+    g.stats.grid = 24;
+    g.stats.items = 24;
+    g.stats.schedule = RT_SCHED_BATCHED;
+    TRY(cudaStreamSynchronize(g.stream));
+    return latched_errors(g);
+  }
   int p = 0;
   TRY(cudaMemcpyAsync(&p, g.src_of_input + src, sizeof(int), cudaMemcpyDeviceToHost, g.stream));
   TRY(cudaStreamSynchronize(g.stream));
   int hitems[24];
   for (int q = 0; q < 24; ++q) hitems[q] = (p << 5) | q;
   TRY(cudaMemcpyAsync(g.queue + 8, hitems, 24 * sizeof(int), cudaMemcpyHostToDevice, g.stream));
-  TRY(launch_precompute(g, false));
-  TRY(cudaMemsetAsync(d_coldens, 0, g.ncell * sizeof(double), g.stream));
   if (schedule == RT_SCHED_PLAIN) {
     hitems[0] = p;
     TRY(cudaMemcpyAsync(g.queue + 8, hitems, sizeof(int), cudaMemcpyHostToDevice, g.stream));
@@ -834,8 +863,7 @@ rt_status rt_iterate(rt_grid_t h, double* d_x, double dt_s, double alpha_H, doub
     double* xin = (k % 2 == 0) ? g.xavg : g.xavg2;
     double* xout = (k % 2 == 0) ? g.xavg2 : g.xavg;
     TRY(launch_one_minus(xin, g.xhi_int, g.ncell, skip, g.stream));
-    TRY(launch_precompute(g, takes_rates_kernels(g), skip));
-    TRY(launch_zero(d_gamma, g.ncell, skip, g.stream));
+    TRY(launch_precompute(g, takes_rates_kernels(g) ? PRE_THICK : PRE_INVN, d_gamma, skip));
     TRY(cudaMemsetAsync(g.unconv, 0, sizeof(int64_t), g.stream));
     if (g.nsrc > 0) {
       rt_status s2 = run_trace(g, d_gamma, nullptr, g.items, 24 * g.nsrc, RT_SCHED_BATCHED, g.nsrc, skip);
@@ -926,8 +954,7 @@ rt_status rt_raytrace_backward(rt_grid_t h, const double* d_dL_dgamma, double* d
   if (g.interp_mode != RT_INTERP_GEOMETRIC)
     return fail(RT_ERR_INVALID, "rt_raytrace_backward: the adjoint is built for the geometric "
                                 "weights (rt_set_interpolation mode 0)");
-  TRY(launch_precompute(g, false));
-  TRY(cudaMemsetAsync(d_dL_dlog_nHI, 0, g.ncell * sizeof(double), g.stream));
+  TRY(launch_precompute(g, PRE_INVN, d_dL_dlog_nHI));
   if (g.nsrc == 0) return RT_OK;
   if (g.dq_cap < g.nsrc) {
     dev_free(g.dq_merged);

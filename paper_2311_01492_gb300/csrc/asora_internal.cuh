@@ -88,6 +88,7 @@ struct TraceArgs {
   const double* ndot;
   const int* r2lim;      // floor(R^2) per source
   const int* items;      // (source << 5) | (face << 2) | quadrant, LPT order
+  const int* one_src;    // rates.cu, column densities: the source (in LPT order)
   int item_begin;        // first item of this launch (the queue counts from here)
   int n_items;           // one past the last item of this launch
   int* queue;            // work counter
@@ -297,11 +298,14 @@ rt_status fail(rt_status st, const std::string& msg);
 rt_status cuda_fail(cudaError_t e, const char* what);
 
 // launchers (defined in the kernel translation units)
-// dtau, its rotated copy, and 1/n_HI or (for the batched rates: thick) zeros in g.invn
-cudaError_t launch_precompute(Grid& g, bool thick, const int* skip = nullptr);
+// dtau, its rotated copy and, in g.invn, what the call needs: 1/n_HI, zeros (the thick
+// sums of the batched rates) or nothing; zeroes `out` (ncell doubles) if not null
+enum { PRE_INVN = 0, PRE_THICK = 1, PRE_DTAU = 2 };
+cudaError_t launch_precompute(Grid& g, int what, double* out, const int* skip = nullptr);
+// coldens /= sigma0 where it is not zero
+cudaError_t launch_tau_to_coldens(Grid& g, double* coldens);
 // gamma += thick / n_HI where thick != 0
 cudaError_t launch_add_thick(Grid& g, double* gamma, const int* skip);
-cudaError_t launch_zero(double* p, int64_t n, const int* skip, cudaStream_t s);
 cudaError_t launch_validate_fields(Grid& g, const double* nH, const double* xHI);
 cudaError_t launch_geometry(GeoEntry* geo, GeoRow* georow, double* kap, double2* binom, int mmax,
                             cudaStream_t s);
@@ -313,7 +317,10 @@ size_t faces_smem_bytes(int hcap, int block, bool od = false);
 int faces_max_grid(int block, size_t smem, int wpb = 8, bool od = false);
 int shells_max_grid(int block);
 // batched rates with the geometric weights (rates.cu); mode: quadrants per warp (1, 2)
-// or 4 for whole faces (wpb warps per CTA), or threads of a CTA (128, 256)
+// or 4 for whole faces (wpb warps per CTA), or threads of a CTA (128, 256; with kAhead
+// 128, 256 or 512, one CTA per item); with a.coldens (kAhead only): the column densities
+// of source *a.one_src
+constexpr int kAhead = 1 << 12;
 cudaError_t launch_rates(Grid& g, const TraceArgs& a, int mode, int grid, size_t smem, int wpb);
 size_t rates_smem_bytes(int hcap, int mode);  // per CTA (warp modes: per warp)
 int rates_max_grid(int mode, size_t smem, int wpb, bool exit);

@@ -45,14 +45,17 @@ cudaError_t launch_validate_fields(Grid& g, const double* nH, const double* xHI)
 // copy dtauT[k][i][j] so that the z faces read rows of constant k contiguously.
 // n_H is the proper density: the given (comoving) one times inv_a3 = a^-3 in an
 // expanding background (inv_a3 = 1 otherwise, an exact no-op); cell (in the
-// box records) is the proper cell size.  THICK: zeros instead of 1/n_HI (the batched
-// rates divide their summed thick terms by n_HI once per cell, k_add_thick; an FP64
-// division per cell made this kernel 2.4 times its memory time at 250^3).
-template <bool THICK>
+// box records) is the proper cell size.  WHAT: 1/n_HI only where it is read; the batched
+// rates divide their summed thick terms by n_HI once per cell (k_add_thick) and take
+// zeros to sum into, column densities need neither (an FP64 division per cell made this
+// kernel 2.4 times its memory time at 250^3).  The call's output field is zeroed here
+// too: one launch less.
+template <int WHAT>
 __global__ void k_precompute(const BoxDev* __restrict__ boxes, const double* __restrict__ nH,
                              const double* __restrict__ xHI, double inv_a3,
                              double* __restrict__ dtau, double* __restrict__ dtauT,
-                             double* __restrict__ invn, const int* __restrict__ skip) {
+                             double* __restrict__ invn, double* __restrict__ out,
+                             const int* __restrict__ skip) {
   __shared__ double tile[32][33];
   if (skip && *skip) return;
   const BoxDev B = boxes[blockIdx.z];
@@ -70,7 +73,9 @@ __global__ void k_precompute(const BoxDev* __restrict__ boxes, const double* __r
         const double nh = nH[idx] * inv_a3, x = xHI[idx];
         const double d = (B.sig_cell * nh) * x;
         dtau[idx] = d;
-        invn[idx] = THICK ? 0.0 : 1.0 / (nh * x);
+        if (WHAT == PRE_INVN) invn[idx] = 1.0 / (nh * x);
+        if (WHAT == PRE_THICK) invn[idx] = 0.0;
+        if (out) out[idx] = 0.0;
         tile[yy][tx] = d;
       }
     }
@@ -84,15 +89,30 @@ __global__ void k_precompute(const BoxDev* __restrict__ boxes, const double* __r
   }
 }
 
-cudaError_t launch_precompute(Grid& g, bool thick, const int* skip) {
+cudaError_t launch_precompute(Grid& g, int what, double* out, const int* skip) {
   const int n = g.nmax;
   dim3 grid((n + 31) / 32, (unsigned)std::min<int64_t>(((int64_t)n * n + 31) / 32, 65535), g.nbox);
-  if (thick)
-    k_precompute<true><<<grid, dim3(32, 8), 0, g.stream>>>(g.boxes_d, g.nH, g.xHI, g.inv_a3, g.dtau,
-                                                           g.dtauT, g.invn, skip);
-  else
-    k_precompute<false><<<grid, dim3(32, 8), 0, g.stream>>>(g.boxes_d, g.nH, g.xHI, g.inv_a3, g.dtau,
-                                                            g.dtauT, g.invn, skip);
+  auto* k = what == PRE_INVN ? k_precompute<PRE_INVN>
+                             : what == PRE_THICK ? k_precompute<PRE_THICK> : k_precompute<PRE_DTAU>;
+  k<<<grid, dim3(32, 8), 0, g.stream>>>(g.boxes_d, g.nH, g.xHI, g.inv_a3, g.dtau, g.dtauT, g.invn,
+                                        out, skip);
+  count_launch();
+  return cudaGetLastError();
+}
+
+// Optical depths to column densities (division: the quotient is rounded once), for the
+// traced part only.
+__global__ void k_tau_to_coldens(int64_t n, double sigma0, double* __restrict__ c) {
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const double v = c[t];
+    if (v != 0.0) c[t] = v / sigma0;
+  }
+}
+
+cudaError_t launch_tau_to_coldens(Grid& g, double* coldens) {
+  const int grid = (int)std::min<int64_t>((g.ncell + 255) / 256, 152 * 16);
+  k_tau_to_coldens<<<grid, 256, 0, g.stream>>>(g.ncell, g.p.sigma0_cm2, coldens);
   count_launch();
   return cudaGetLastError();
 }
@@ -112,20 +132,6 @@ __global__ void k_add_thick(int64_t n, const double* __restrict__ nH, const doub
 cudaError_t launch_add_thick(Grid& g, double* gamma, const int* skip) {
   const int grid = (int)std::min<int64_t>((g.ncell + 255) / 256, 152 * 16);
   k_add_thick<<<grid, 256, 0, g.stream>>>(g.ncell, g.nH, g.xHI, g.inv_a3, g.invn, gamma, skip);
-  count_launch();
-  return cudaGetLastError();
-}
-
-__global__ void k_zero(double* __restrict__ p, int64_t n, const int* __restrict__ skip) {
-  if (skip && *skip) return;
-  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n;
-       c += (int64_t)gridDim.x * blockDim.x)
-    p[c] = 0.0;
-}
-
-cudaError_t launch_zero(double* p, int64_t n, const int* skip, cudaStream_t s) {
-  const int grid = (int)std::min<int64_t>((n + 255) / 256, 152 * 8);
-  k_zero<<<grid, 256, 0, s>>>(p, n, skip);
   count_launch();
   return cudaGetLastError();
 }

@@ -69,12 +69,16 @@ static size_t rates_cta_bytes(int h, int slots) {
   return 2 * rates_buf_bytes(h) + (size_t)slots * row_slot_bytes(h);
 }
 
-// Row-table slots of a CTA: the current layer's and the next's, or one (the next
-// layer's table then waits for the end of the layer) where two do not fit.
-static int cta_slots(int h) { return rates_cta_bytes(h, 2) <= 227 * 1024 ? 2 : 1; }
+// Row-table slots of a CTA: this layer's and those staged ahead, or one (the next layer's
+// table then waits for the end of the layer) where they do not fit.
+static int cta_slots(int h, bool ahead) {
+  const int n = ahead ? 3 : 2;
+  return rates_cta_bytes(h, n) <= 227 * 1024 ? n : 1;
+}
 
 size_t rates_smem_bytes(int hcap, int mode) {
-  return mode <= 4 ? rates_warp_bytes(hcap, mode) : rates_cta_bytes(hcap, cta_slots(hcap));
+  return mode <= 4 ? rates_warp_bytes(hcap, mode)
+                   : rates_cta_bytes(hcap, cta_slots(hcap, mode & kAhead));
 }
 
 // ----------------------------------------------------------------- quadrants
@@ -91,6 +95,7 @@ struct Quad {
   const double* fld;       // dtau, rotated for the z faces: the stride of a2 is 1
 };
 
+template <bool RATED = true>
 __device__ __forceinline__ Quad quad_setup(const TraceArgs& a, const int item, const bool first,
                                            unsigned& nrate) {
   Quad Q;
@@ -112,7 +117,8 @@ __device__ __forceinline__ Quad quad_setup(const TraceArgs& a, const int item, c
   Q.half_dts = 0.5 * a.dtau[scell];
   Q.nd_thick = nd * B.inv_cell3;
   Q.nd_thin = nd * B.thin_fac;
-  if (f == 4 && quad == 0 && first) {  // the source cell (q = 0), once per source
+  if (!RATED && f == 4 && quad == 0 && first) a.coldens[scell] = Q.half_dts;
+  if (RATED && f == 4 && quad == 0 && first) {  // the source cell (q = 0), once per source
     double dG;
     if (bits_of(Q.half_dts) <= bits_of(a.tau_lim))
       dG = nd * (tab_eval(a.tab.h, a.tab, 0.0) * (0.5 * B.thin_fac));
@@ -227,6 +233,20 @@ __device__ __forceinline__ void deposit_rate(const TraceArgs& a, const Quad& Q, 
   }
   ++nrate;
   if (dG != 0.0) atomicAdd(&out[cell], dG);
+}
+
+// Optical depth through a cell that a quadrant owns, to its place in C order.
+__device__ __forceinline__ void write_column(const TraceArgs& a, const Quad& Q, const int m,
+                                             const CellIn& c, const double tout) {
+  const bool own = ((Q.d == 2) || (Q.d == 1 ? c.t2 < m : (c.t1 < m && c.t2 < m))) &&
+                   (c.t1 > 0 || Q.q1 > 0) && (c.t2 > 0 || Q.q2 > 0);
+  if (!own) return;
+  int64_t cell = Q.off + c.gidx;
+  if (Q.d == 2) {
+    const int x1 = wrapc(Q.c1 + Q.q1 * c.t1, Q.N), x2 = wrapc(Q.c2 + Q.q2 * c.t2, Q.N);
+    cell = Q.off + (x1 * Q.N + x2) * Q.N + wrapc(Q.cd + Q.sg * m, Q.N);
+  }
+  a.coldens[cell] = tout;
 }
 
 // Doubles of the part of a layer buffer that an item can read before it writes it
@@ -462,105 +482,160 @@ __device__ __forceinline__ void rates_item_warp(const TraceArgs& a, const int it
   }
 }
 
-// One quadrant item by a CTA of GS threads (large sources): two layer buffers and a
-// barrier per layer.
-template <int GS, bool EXIT>
+// One quadrant item by a CTA of GS threads: sources too wide for warps, and whatever has
+// too few items to fill the GPU.  Two layer buffers and a barrier per layer; the row
+// tables are staged one layer ahead.  AHEAD, for launches of few items, where the time
+// of a layer is what counts: tables two layers ahead, so that each thread loads the
+// indices, dtau and weights of its first cell of the next layer before it computes this
+// one (more registers and shared memory than a full GPU has to spare: 128^3, 40 sources
+// of R = 40: 0.21 against 0.12 ms).
+// WHAT: rates, rates with the early exit, or the column densities of one source (as
+// optical depths: launch_tau_to_coldens divides by sigma0 on all SMs).
+enum { RATES = 0, RATES_EXIT = 1, COLDENS = 2 };
+
+template <int GS, int WHAT, bool AHEAD>
 __device__ __forceinline__ void rates_item_cta(const TraceArgs& a, const int item, const int gt,
                                                unsigned char* __restrict__ sm, const int h,
                                                const int slots, unsigned& nrate) {
+  constexpr int D = AHEAD ? 2 : 1;  // layers that the tables are staged ahead (slots == D + 1)
   const int W = h + 2;
   const int TS = row_slot_bytes(h);
   double* cur = reinterpret_cast<double*>(sm);
   double* prev = reinterpret_cast<double*>(sm + rates_buf_bytes(h));
   unsigned char* tab = sm + 2 * rates_buf_bytes(h);
   const int wid = gt >> 5, lane = gt & 31;
-  const Quad Q = quad_setup(a, item, gt == 0, nrate);
+  const Quad Q = quad_setup<WHAT != COLDENS>(a, item, gt == 0, nrate);
   for (int t = gt, n = zero_count(Q.R2, h); t < n; t += GS) cur[t] = prev[t] = 0.0;
-  const int ent = first_layer_entry(a, Q.R2, min(Q.lim1, Q.lim2));
-  auto slot_of = [&](int m) { return tab + (slots == 2 ? (m & 1) * TS : 0); };
+  if (Q.Lmax < 1) return;
+  // tables know no window: cells outside it are left out one by one
+  const int ent = first_layer_entry(a, Q.R2, h);
+  int sq = isqrt_i(Q.R2 - 1);
+  auto half_width = [&](int m) {  // for m ascending
+    while (sq * sq > Q.R2 - m * m) --sq;
+    return min(m, sq);
+  };
+  bool bad = false;
   auto stage = [&](int m, int H) {  // row table of layer m (waited for separately)
-    if (ent >= 0) {
+    unsigned char* dst = tab + (slots > 1 ? m % (D + 1) * TS : 0);
+    if (H > h) {
+      bad = true;
+    } else if (ent >= 0) {
       const int4 lay = __ldg(&a.rtab_lay[ent + m - 1]);
-      stage_rows<GS>(a.rtab + lay.x, lay.y, slot_of(m), gt);
+      stage_rows<GS>(a.rtab + lay.x, lay.y, dst, gt);
     } else if (wid == 0) {
-      const int nr = min(H, Q.lim1) + 1;
-      int* pre = reinterpret_cast<int*>(slot_of(m));
-      quad_rows_warp(Q.R2 - m * m, H, nr, Q.lim2, pre,
-                     reinterpret_cast<unsigned char*>(pre + nr + 1), lane);
+      int* pre = reinterpret_cast<int*>(dst);
+      quad_rows_warp(Q.R2 - m * m, H, H + 1, h, pre,
+                     reinterpret_cast<unsigned char*>(pre + H + 2), lane);
     }
   };
-  if (Q.Lmax >= 1) {
-    const int H1 = min(1, isqrt_i(Q.R2 - 1));
-    if (H1 <= h) stage(1, H1);
-    cp_async_wait_all();
+  struct Layer {
+    const int* rowpre;
+    const unsigned char* rowof;
+    int total, base, gofs;
+  };
+  auto layer = [&](int m, int H) {
+    Layer L;
+    L.rowpre = reinterpret_cast<const int*>(tab + (slots > 1 ? m % (D + 1) * TS : 0));
+    L.rowof = reinterpret_cast<const unsigned char*>(L.rowpre + H + 2);
+    L.total = L.rowpre[H + 1];
+    L.base = wrapc(Q.cd + Q.sg * m, Q.N) * Q.md + Q.org;
+    L.gofs = (int)georow_index(m, 0, 0);
+    return L;
+  };
+  struct Ahead {  // a cell and its weights (scaled part: kappa ds in c.kds)
+    CellIn c;
+    Weights w;
+    const GeoRow* gr;
+  };
+  auto load = [&](Ahead& x, const Layer& L, int m, int t, bool scaled) {
+    fetch_cell(Q, x.c, t, L.base, L.rowpre, L.rowof);
+    const int o = L.gofs + x.c.t1 * (m + 1) + x.c.t2;
+    x.gr = a.georow + o;
+    if (scaled) x.c.kds = __ldg(&a.kap[o]);
+    else x.w = load_weights(x.gr);
+  };
+  bool opaque = true;  // every cell of this thread in the layer has tau_out beyond the bound
+  auto rated = [&](const Ahead& x, int m, double tin) {  // the cell's column, and its rate
+    const double tout = fma(x.c.dtp, x.w.ds, tin);
+    if (x.c.t1 > Q.lim1 || x.c.t2 > Q.lim2) return;
+    cur[(x.c.t1 + 1) * W + x.c.t2 + 1] = tout;
+    if (WHAT == COLDENS) {
+      write_column(a, Q, m, x.c, tout);
+      return;
+    }
+    opaque = opaque && bits_of(tout) >= a.exit_bits;
+    if (bits_of(tin) < a.tab.tau_max_bits)
+      deposit_rate<false>(a, Q, m, x.c, x.gr, x.w.ds, tin, tout, nrate);
+  };
+  int Hc = half_width(1), Hn = 0;  // of this layer and the next
+  stage(1, Hc);
+  if (Q.Lmax > 1) {
+    Hn = half_width(2);
+    if (AHEAD && slots > 1) stage(2, Hn);
   }
+  cp_async_wait_all();
   group_sync<GS>();
-  bool scaled = false;
+  bool scaled = false, ahead_scaled = false;
+  Ahead nx;
   for (int m = 1; m <= Q.Lmax; ++m) {
-    const int H = min(m, isqrt_i(Q.R2 - m * m));
-    if (H > h || m > a.kap_mmax) {
-      if (gt == 0) atomicOr(a.err, H > h ? ERR_LAYER_CAP : ERR_GEO);
+    if (bad || m > a.kap_mmax) {  // (a layer found too wide when it was to be staged)
+      if (gt == 0) atomicOr(a.err, bad ? ERR_LAYER_CAP : ERR_GEO);
       break;
     }
-    const int nrows = min(H, Q.lim1) + 1;
-    const int* rowpre = reinterpret_cast<const int*>(slot_of(m));
-    const unsigned char* rowof = reinterpret_cast<const unsigned char*>(rowpre + nrows + 1);
-    const int total = rowpre[nrows];
-    int Hn = 0;  // half-width of the next layer
-    if (m < Q.Lmax) {
-      Hn = min(m + 1, isqrt_i(Q.R2 - (m + 1) * (m + 1)));
-      if (slots == 2 && Hn <= h && ent >= 0) stage(m + 1, Hn);
+    const Layer L = layer(m, Hc);
+    int Hnn = 0;
+    if (m + 2 <= Q.Lmax) Hnn = half_width(m + 2);
+    if (slots > 1 && m + D <= Q.Lmax) stage(m + D, AHEAD ? Hnn : Hn);
+    Ahead x = nx;
+    const bool have = AHEAD && slots > 1 && m > 1;  // x: this thread's first cell
+    bool x_scaled = ahead_scaled;
+    if (AHEAD && slots > 1 && m < Q.Lmax && Hn <= h) {
+      const Layer Ln = layer(m + 1, Hn);
+      if (gt < Ln.total) load(nx, Ln, m + 1, gt, scaled);
+      ahead_scaled = scaled;
     }
-    const int base = wrapc(Q.cd + Q.sg * m, Q.N) * Q.md + Q.org;
-    const int gofs = (int)georow_index(m, 0, 0);
-    bool opaque = true;  // every cell of this thread has tau_out beyond the bound
-    CellIn c;
-    if (scaled) {
-      for (int t = gt; t < total; t += GS) {
-        fetch_cell(Q, c, t, base, rowpre, rowof);
-        const double kds = __ldg(&a.kap[gofs + c.t1 * (m + 1) + c.t2]);
-        const int o = (c.t1 + 1) * W + c.t2 + 1;
-        const double* s = prev + o;
-        cur[o] = fma(c.dtp, kds, bracket_sum(s[0], s[-W], s[-1], s[-W - 1]));
+    opaque = true;
+    if (m == 1) {  // the column from the source centre to the layer's entry plane
+      if (gt < L.total) {
+        load(x, L, m, gt, false);
+        rated(x, m, Q.half_dts * x.w.ds);
       }
     } else {
-      auto cells = [&](auto first) {
-        constexpr bool FIRST = decltype(first)::value;
-        for (int t = gt; t < total; t += GS) {
-          fetch_cell(Q, c, t, base, rowpre, rowof);
-          const GeoRow* gr = a.georow + gofs + c.t1 * (m + 1) + c.t2;
-          const int o = (c.t1 + 1) * W + c.t2 + 1;
-          const Weights w = load_weights(gr);
-          double tin;
-          if constexpr (FIRST) tin = Q.half_dts * w.ds;
-          else tin = interp(a, w, prev + o, W, 1);
-          const double tout = fma(c.dtp, w.ds, tin);
-          cur[o] = tout;
-          opaque = opaque && bits_of(tout) >= a.exit_bits;
-          if (bits_of(tin) < a.tab.tau_max_bits)
-            deposit_rate<false>(a, Q, m, c, gr, w.ds, tin, tout, nrate);
+      for (int t = gt; t < L.total; t += GS) {
+        if (t > gt || !have) {
+          load(x, L, m, t, scaled);
+          x_scaled = scaled;
         }
-      };
-      if (m == 1) cells(std::true_type());
-      else cells(std::false_type());
+        const double* s = prev + (x.c.t1 + 1) * W + x.c.t2 + 1;
+        if (scaled) {
+          if (AHEAD && !x_scaled) x.c.kds = __ldg(&a.kap[x.gr - a.georow]);  // (loaded for a rated layer)
+          const double v = fma(x.c.dtp, x.c.kds, bracket_sum(s[0], s[-W], s[-1], s[-W - 1]));
+          if (x.c.t1 <= Q.lim1 && x.c.t2 <= Q.lim2) cur[(x.c.t1 + 1) * W + x.c.t2 + 1] = v;
+        } else {
+          rated(x, m, interp(a, x.w, s, W, 1));
+        }
+      }
     }
-    if (m < Q.Lmax && Hn <= h) {  // row table of the next layer
-      if (slots == 1) group_sync<GS>();  // this layer's is no longer read
-      if (slots == 1 || ent < 0) stage(m + 1, Hn);
-      cp_async_wait_all();
+    if (slots == 1 && m < Q.Lmax) {
+      group_sync<GS>();  // this layer's table is no longer read
+      stage(m + 1, Hn);
     }
-    if (scaled) {
-      group_sync<GS>();
+    cp_async_wait_all();
+    if (WHAT == COLDENS || scaled) {
+      __syncthreads();
     } else if (__syncthreads_and(opaque)) {  // as in rates_item_warp
-      if (EXIT) break;
+      if (WHAT == RATES_EXIT) break;
       scaled = true;
       scale_layer<GS>(a, cur, W, m, h, gt);
-      group_sync<GS>();
+      __syncthreads();
     }
     double* tmp = prev;
     prev = cur;
     cur = tmp;
+    Hc = Hn;
+    Hn = Hnn;
   }
+  cp_async_wait_all();
 }
 
 __device__ __forceinline__ void flush_rates(const TraceArgs& a, unsigned nrate) {
@@ -569,21 +644,29 @@ __device__ __forceinline__ void flush_rates(const TraceArgs& a, unsigned nrate) 
   if ((threadIdx.x & 31) == 0 && nrate) atomicAdd(a.rate_cells, (unsigned long long)nrate);
 }
 
-template <int BLOCK, bool EXIT>
-__global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) k_rates_cta(TraceArgs a, int slots) {
+template <int BLOCK, int WHAT, bool AHEAD>
+__global__ void __launch_bounds__(BLOCK, (AHEAD ? 512 : 1024) / BLOCK) k_rates_cta(TraceArgs a,
+                                                                                int slots) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_item;
   if (a.skip && *a.skip) return;
   unsigned nrate = 0;
-  for (;;) {
-    __syncthreads();
-    if (threadIdx.x == 0) s_item = a.item_begin + atomicAdd(a.queue, 1);
-    __syncthreads();
-    const int it = s_item;
-    if (it >= a.n_items) break;
-    rates_item_cta<BLOCK, EXIT>(a, a.items[it], threadIdx.x, smem_raw, a.hcap, slots, nrate);
+  if (AHEAD) {  // as many CTAs as there are items
+    const int item = WHAT == COLDENS ? (*a.one_src << 5) | (int)blockIdx.x
+                                     : a.items[a.item_begin + blockIdx.x];
+    rates_item_cta<BLOCK, WHAT, AHEAD>(a, item, threadIdx.x, smem_raw, a.hcap, slots, nrate);
+  } else {
+    for (;;) {
+      __syncthreads();
+      if (threadIdx.x == 0) s_item = a.item_begin + atomicAdd(a.queue, 1);
+      __syncthreads();
+      const int it = s_item;
+      if (it >= a.n_items) break;
+      rates_item_cta<BLOCK, WHAT, AHEAD>(a, a.items[it], threadIdx.x, smem_raw, a.hcap, slots,
+                                         nrate);
+    }
   }
-  flush_rates(a, nrate);
+  if (WHAT != COLDENS) flush_rates(a, nrate);
 }
 
 template <int MODE, bool EXIT>
@@ -604,29 +687,48 @@ __global__ void __launch_bounds__(256, 2) k_rates_warp(TraceArgs a) {
   flush_rates(a, nrate);
 }
 
-// mode: quadrants per warp (1, 2), 4: a whole face per warp, or threads of a CTA (128, 256)
-static const void* rates_kernel(int mode, bool exit) {
-#define ASORA_PICK(...) (exit ? (const void*)__VA_ARGS__, true> : (const void*)__VA_ARGS__, false>)
+// mode: quadrants per warp (1, 2), 4: a whole face per warp, or threads of a CTA (128,
+// 256; with kAhead 128, 256, 512)
+static const void* rates_kernel(int mode, int what) {
+#define ASORA_PICK(K, ...)                                                \
+  (what == RATES_EXIT ? (const void*)K<__VA_ARGS__ RATES_EXIT ASORA_REST> \
+                      : (const void*)K<__VA_ARGS__ RATES ASORA_REST>)
+#define ASORA_REST
   switch (mode) {
-    case 1: return ASORA_PICK(k_rates_warp<1);
-    case 2: return ASORA_PICK(k_rates_warp<2);
-    case 4: return ASORA_PICK(k_rates_warp<4);
-    case 128: return ASORA_PICK(k_rates_cta<128);
-    case 256: return ASORA_PICK(k_rates_cta<256);
+    case 1: return ASORA_PICK(k_rates_warp, 1, );
+    case 2: return ASORA_PICK(k_rates_warp, 2, );
+    case 4: return ASORA_PICK(k_rates_warp, 4, );
+#undef ASORA_REST
+#define ASORA_REST , false
+    case 128: return ASORA_PICK(k_rates_cta, 128, );
+    case 256: return ASORA_PICK(k_rates_cta, 256, );
+#undef ASORA_REST
+#define ASORA_REST , true
+    case 128 | kAhead:
+      return what == COLDENS ? (const void*)k_rates_cta<128, COLDENS, true>
+                             : ASORA_PICK(k_rates_cta, 128, );
+    case 256 | kAhead:
+      return what == COLDENS ? (const void*)k_rates_cta<256, COLDENS, true>
+                             : ASORA_PICK(k_rates_cta, 256, );
+    case 512 | kAhead:
+      return what == COLDENS ? (const void*)k_rates_cta<512, COLDENS, true>
+                             : ASORA_PICK(k_rates_cta, 512, );
     default: return nullptr;
   }
+#undef ASORA_REST
 #undef ASORA_PICK
 }
 
 cudaError_t launch_rates(Grid& g, const TraceArgs& a, int mode, int grid, size_t smem, int wpb) {
-  const void* fn = rates_kernel(mode, a.early_exit != 0);
+  const void* fn =
+      rates_kernel(mode, a.coldens ? COLDENS : a.early_exit ? RATES_EXIT : RATES);
   if (!fn) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   TraceArgs arg = a;
-  int slots = mode <= 4 ? 2 : cta_slots(a.hcap);
-  void* params[] = {&arg, &slots};
-  e = cudaLaunchKernel(fn, dim3(grid), dim3(mode <= 4 ? wpb * 32 : mode), params, smem, g.stream);
+  int slots = cta_slots(a.hcap, mode & kAhead);
+  void* params[] = {&arg, &slots};  // (the warp kernels take the first only)
+  e = cudaLaunchKernel(fn, dim3(grid), dim3(mode <= 4 ? wpb * 32 : mode & ~kAhead), params, smem, g.stream);
   count_launch();
   return e;
 }
@@ -635,11 +737,12 @@ int rates_max_grid(int mode, size_t smem, int wpb, bool exit) {
   int dev = 0, sms = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const void* fn = rates_kernel(mode, exit);
+  const void* fn = rates_kernel(mode, exit ? RATES_EXIT : RATES);
   if (!fn) return 0;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, mode <= 4 ? wpb * 32 : mode, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, mode <= 4 ? wpb * 32 : mode & ~kAhead,
+                                                      smem);
   if (e != cudaSuccess) return 0;
   return per * sms;
 }
