@@ -91,7 +91,7 @@ static void free_grid(Grid* g) {
   dev_free(g->geo); dev_free(g->georow); dev_free(g->kap); dev_free(g->queue); dev_free(g->err);
   dev_free(g->cube); dev_free(g->unconv); dev_free(g->xbuf); dev_free(g->xavg);
   dev_free(g->xavg2); dev_free(g->xhi_int); dev_free(g->flags); dev_free(g->counters);
-  dev_free(g->bwd_stack); dev_free(g->dq_merged);
+  dev_free(g->bwd_stack); dev_free(g->dq_merged); dev_free(g->bwd_redo);
   free_row_tables(*g);
   if (g->it_exec) cudaGraphExecDestroy(g->it_exec);
   if (g->it_stream) cudaStreamDestroy(g->it_stream);
@@ -123,7 +123,7 @@ static rt_status ensure_geometry(Grid& g, int mmax) {
   double* kap = nullptr;
   double2* binom = nullptr;
   cudaError_t e = dev_malloc(&georow, georow_count(mmax) * sizeof(GeoRow));
-  if (e == cudaSuccess) e = dev_malloc(&kap, 2 * georow_count(kmax) * sizeof(double));
+  if (e == cudaSuccess) e = dev_malloc(&kap, 3 * georow_count(kmax) * sizeof(double));
   if (e == cudaSuccess) e = dev_malloc(&binom, (size_t)(kmax + 1) * (kmax + 2) / 2 * sizeof(double2));
   if (e == cudaSuccess) e = launch_geometry(geo, georow, kap, binom, mmax, g.stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(g.stream);  // binom is still read
@@ -184,6 +184,7 @@ static TraceArgs base_args(Grid& g) {
   a.kap = g.kap;
   a.kap_mmax = g.kap_mmax;
   a.kappa = g.kap ? g.kap + georow_count(g.kap_mmax) : nullptr;
+  a.ikappa = g.kap ? g.kap + 2 * georow_count(g.kap_mmax) : nullptr;
   a.tab.g = g.gtab;
   a.tab.h = g.htab;
   a.tab.kind = g.tab_kind;
@@ -275,6 +276,17 @@ static int first_fitting(const Grid& g, const int* r2s, int ns, int hlim) {
 // 168 / 137 / 133; 223 / 176 / 169; R = 70 (49) 566 / 382 / 321; 881 / 537 / 454.
 static int few_items_block(int h) { return (h < 12 ? 128 : h < 24 ? 256 : 512) | kAhead; }
 
+// How much longer a warp would take for one of `parts` equal parts of the widest source's
+// ball than all work takes the GPU's resident warps (16 per SM at the larger widths).
+static double longest_part(const Grid& g, int parts) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const double r = std::sqrt((double)g.max_r2);
+  const double ball = std::min(4.18879 * r * r * r, (double)g.nmax * g.nmax * g.nmax);
+  return ball / parts * (16.0 * sms) / std::max(1.0, (double)g.source_voxels);
+}
+
 // Launches of the batched rates: sources [cut[k], cut[k+1]) (LPT order) by CTAs of
 // mode[0] threads (k = 0) or by warps with one quadrant, two, or a whole face (k = 1..3).
 struct RatesPlan {
@@ -308,10 +320,8 @@ static RatesPlan rates_plan(const Grid& g, const int* r2s, int ns) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const double warps = 16.0 * sms;  // resident at the larger half-widths
-  const double r = std::sqrt((double)r2s[0]);
-  const double ball = std::min(4.18879 * r * r * r, (double)g.nmax * g.nmax * g.nmax);
   p.mode[0] = 128;
-  if (ball * warps > 1.2 * 24 * (double)g.source_voxels) {
+  if (longest_part(g, 24) > 1.2) {
     const int h = face_hcap(r2s[0], g.nmax);
     if (24 * ns <= 2 * sms) p.mode[0] = few_items_block(h);
     else if (24 * ns <= 4 * sms && h >= 24) p.mode[0] = 256;
@@ -964,47 +974,72 @@ rt_status rt_raytrace_backward(rt_grid_t h, const double* d_dL_dgamma, double* d
     g.dq_cap = g.nsrc;
   }
   TRY(cudaMemsetAsync(g.dq_merged, 0, g.nsrc * sizeof(double), g.stream));
-  // items of large sources by 128-thread CTAs, the rest one per warp (as the trace,
-  // but with the warp-mode threshold capped at half-width 27: an adjoint warp keeps
-  // two layers and its layer records in shared memory, and beyond 27 too few of
-  // its warps stay resident -- 1e5 sources of the 250^3 workload took 1.5x longer
-  // at 30)
+  // Whole faces by warps (k_bwd_faces): every source if the recompute may stop at opaque
+  // layers (what does not fit is left to the quadrant kernels, through a list on the
+  // device), else those whose layers all fit.  Quadrant items of large sources by
+  // 128-thread CTAs, the rest one per warp (as the trace, but with the warp-mode threshold
+  // capped at half-width 27: such a warp keeps two layers and its layer records in shared
+  // memory, and beyond 27 too few stay resident -- 1e5 sources of the 250^3 workload took
+  // 1.5x longer at 30).
+  const int ns = g.nsrc;
+  const int* r2s = g.r2_sorted_h.data();
   const int hbig = face_hcap(g.max_r2, g.nmax);
   const int lcap = std::max(1, std::min(isqrt_h(g.max_r2), g.nmax / 2 + 1));
-  const int n_items = 24 * g.nsrc;
-  const int hsmall_bwd = std::min(g.hsmall, 27);
-  int split = n_items, hsm = 0, r2sm = 0;
-  if (hsmall_bwd > 0 && !g.r2_sorted_h.empty()) {
-    int lo = 0, hi = (int)g.r2_sorted_h.size();
-    while (lo < hi) {
-      const int mid = (lo + hi) / 2;
-      if (face_hcap(g.r2_sorted_h[mid], g.nmax) <= hsmall_bwd) hi = mid; else lo = mid + 1;
-    }
-    if (lo < (int)g.r2_sorted_h.size()) {
-      split = 24 * lo;
-      hsm = face_hcap(g.r2_sorted_h[lo], g.nmax);
-      r2sm = g.r2_sorted_h[lo];
-    }
-  }
-  size_t smem_c = 0, smem_w = 0, cap_c = 0, cap_w = 0;
-  int grid_c = 0, grid_w = 0;
+  const bool exit = g.bwd_exit != 0;
+  // Few items: the longest face decides (1e3 sources of R = 22, ms: faces 0.99, quadrants
+  // 0.51; 4e3 of R = 5..50: 2.18, 2.09; 1e5: 41.8, 55); fewer still, CTAs take every
+  // quadrant (64^3, 256 sources: CTAs 0.21, with warps 0.47).
+  const bool tables = g.ftab && g.kap_mmax >= 1 && longest_part(g, 6) <= 0.3;
+  const int hwarp = !g.explicit_schedule && longest_part(g, 24) > 1.2 ? 0 : std::min(g.hsmall, 27);
+  const int face_begin = !tables ? ns : exit ? 0 : first_fitting(g, r2s, ns, kBwdFaceHcap);
+  const bool leftover = tables && exit && hbig > kBwdFaceHcap;
+  const int quads = exit && tables ? (leftover ? ns : 0) : face_begin;  // sources of the quadrant kernels
+  const int split = std::min(quads, first_fitting(g, r2s, ns, hwarp));
+  BwdLaunch Lc, Lw, Lf;  // CTAs, warps, faces
+  Lc.exit = Lw.exit = Lf.exit = exit;
+  Lc.lcap = Lw.lcap = lcap;
   if (split > 0) {
-    smem_c = bwd_smem_bytes(hbig, lcap);
-    if (smem_c > 227 * 1024)
+    Lc.block = 128;
+    Lc.smem = bwd_smem_bytes(hbig, lcap);
+    if (Lc.smem > 227 * 1024)
       return fail(RT_ERR_INVALID, "rt_raytrace_backward: radius too large for the shared-memory layers");
-    cap_c = face_stack_cap(g.max_r2, g.nmax);
-    const int maxg = bwd_max_grid(smem_c, 128);
+    Lc.stack_cap = face_stack_cap(g.max_r2, g.nmax);
+    const int maxg = bwd_max_grid(Lc.smem, 128);
     if (maxg <= 0) return fail(RT_ERR_CUDA, "rt_raytrace_backward: no occupancy");
-    grid_c = std::max(1, std::min(split, maxg));
+    Lc.grid = std::max(1, std::min(24 * split, maxg));
   }
-  if (split < n_items) {
-    smem_w = bwd_smem_bytes(hsm, lcap) * 8;
-    cap_w = face_stack_cap(r2sm, g.nmax);
-    const int maxg = bwd_max_grid(smem_w, 32);
+  const int hw = split < quads ? face_hcap(r2s[split], g.nmax) : 0;
+  if (split < quads) {
+    Lw.block = 32;
+    Lw.smem = bwd_smem_bytes(hw, lcap) * 8;
+    Lw.stack_cap = face_stack_cap(r2s[split], g.nmax);
+    const int maxg = bwd_max_grid(Lw.smem, 32);
     if (maxg <= 0) return fail(RT_ERR_CUDA, "rt_raytrace_backward: no occupancy (warp mode)");
-    grid_w = std::max(1, std::min((n_items - split + 7) / 8, maxg));
+    Lw.grid = std::max(1, std::min((24 * (quads - split) + 7) / 8, maxg));
   }
-  const size_t need = (cap_c * (size_t)grid_c + cap_w * (size_t)grid_w * 8) * sizeof(double2);
+  const int hf = std::min(hbig, kBwdFaceHcap);
+  const int nfaces = 6 * (ns - face_begin);
+  if (nfaces > 0) {
+    Lf.block = 4;
+    Lf.stack_cap = (size_t)std::max(g.face_stack, 1);
+    int maxg = 0;
+    Lf.wpb = 1;
+    for (int cand = 8; cand >= 1; --cand) {
+      const int mg = bwd_max_grid(bwd_face_smem_bytes(hf) * cand, 4, cand);
+      if (mg * cand > maxg * Lf.wpb) {
+        maxg = mg;
+        Lf.wpb = cand;
+      }
+    }
+    if (maxg <= 0) return fail(RT_ERR_CUDA, "rt_raytrace_backward: no occupancy (faces)");
+    Lf.smem = bwd_face_smem_bytes(hf) * Lf.wpb;
+    Lf.grid = std::max(1, std::min((nfaces + Lf.wpb - 1) / Lf.wpb, maxg));
+    Lf.redo_cap = leftover ? 24 * ns : 0;
+    Lf.split_src = split;
+  }
+  const size_t stack_c = Lc.stack_cap * Lc.grid, stack_w = Lw.stack_cap * Lw.grid * 8;
+  const size_t stack_f = Lf.stack_cap * Lf.grid * Lf.wpb;  // (before the others, in their place)
+  const size_t need = std::max(stack_c + stack_w, stack_f) * sizeof(double2);
   if (need > g.bwd_stack_bytes) {
     dev_free(g.bwd_stack);
     g.bwd_stack = nullptr;
@@ -1012,37 +1047,48 @@ rt_status rt_raytrace_backward(rt_grid_t h, const double* d_dL_dgamma, double* d
     TRY(dev_malloc(&g.bwd_stack, need));
     g.bwd_stack_bytes = need;
   }
+  if (leftover && (size_t)Lf.redo_cap * 2 > g.bwd_redo_cap) {
+    dev_free(g.bwd_redo);
+    g.bwd_redo = nullptr;
+    g.bwd_redo_cap = 0;
+    TRY(dev_malloc(&g.bwd_redo, (size_t)Lf.redo_cap * 2 * sizeof(int)));
+    g.bwd_redo_cap = (size_t)Lf.redo_cap * 2;
+  }
   TraceArgs a = base_args(g);
   a.items = g.items;
-  TRY(cudaMemsetAsync(g.queue, 0, 2 * sizeof(int), g.stream));
+  // queue: [0] CTAs, [1] warps, [2] faces, [4], [5] items left over for the first two
+  TRY(cudaMemsetAsync(g.queue, 0, 6 * sizeof(int), g.stream));
   TRY(cudaEventRecord(g.ev[1], g.stream));
   g.stats.launches = 0;
-  if (split > 0) {
+  auto launch = [&](BwdLaunch& L, int hcap, int begin, int end, int* queue, double2* stack) {
     TraceArgs b = a;
-    b.hcap = hbig;
-    b.item_begin = 0;
-    b.n_items = split;
-    b.queue = g.queue;
-    TRY(launch_trace_bwd(g, b, d_dL_dgamma, d_dL_dlog_nHI, g.dq_merged, g.bwd_stack, cap_c, lcap,
-                         grid_c, smem_c, 128, g.bwd_exit != 0));
+    b.hcap = hcap;
+    b.item_begin = begin;
+    b.n_items = end;
+    b.queue = queue;
+    if (L.n_dev) b.items = L.redo;
     g.stats.launches += 1;
+    return launch_trace_bwd(g, b, L, d_dL_dgamma, d_dL_dlog_nHI, g.dq_merged, stack);
+  };
+  if (nfaces > 0) {
+    Lf.redo = g.bwd_redo;
+    Lf.redo_n = g.queue + 4;
+    TRY(launch(Lf, hf, 6 * face_begin, 6 * ns, g.queue + 2, g.bwd_stack));
   }
-  if (split < n_items) {
-    TraceArgs b = a;
-    b.hcap = hsm;
-    b.item_begin = split;
-    b.n_items = n_items;
-    b.queue = g.queue + 1;
-    TRY(launch_trace_bwd(g, b, d_dL_dgamma, d_dL_dlog_nHI, g.dq_merged,
-                         g.bwd_stack + cap_c * (size_t)grid_c, cap_w, lcap, grid_w, smem_w, 32,
-                         g.bwd_exit != 0));
-    g.stats.launches += 1;
+  if (leftover) {
+    Lc.redo = g.bwd_redo;
+    Lc.n_dev = g.queue + 4;
+    Lw.redo = g.bwd_redo + Lf.redo_cap;
+    Lw.n_dev = g.queue + 5;
   }
+  if (split > 0) TRY(launch(Lc, hbig, 0, 24 * split, g.queue, g.bwd_stack));
+  if (split < quads)
+    TRY(launch(Lw, hw, leftover ? 0 : 24 * split, 24 * quads, g.queue + 1, g.bwd_stack + stack_c));
   TRY(cudaEventRecord(g.ev[2], g.stream));
   TRY(launch_dndot_inputs(g, g.dq_merged, d_dL_dlog_ndot));
-  g.stats.block = split > 0 ? 128 : 32;
-  g.stats.grid = split > 0 ? grid_c : grid_w;
-  g.stats.items = n_items;
+  g.stats.block = nfaces > 0 ? 32 * Lf.wpb : split > 0 ? 128 : 32;
+  g.stats.grid = nfaces > 0 ? Lf.grid : split > 0 ? Lc.grid : Lw.grid;
+  g.stats.items = 24 * ns;
   return RT_OK;
 }
 

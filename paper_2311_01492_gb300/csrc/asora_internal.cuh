@@ -65,6 +65,8 @@ constexpr int kKapMax = 200;
 // Largest layer half-width with face tables (the largest that rt_set_schedule accepts
 // for whole faces).
 constexpr int kFaceHcap = 20;
+// Layer half-width that the adjoint's whole faces have room for.
+constexpr int kBwdFaceHcap = 16;
 
 // Rate tables on the device.
 struct TabDev {
@@ -97,6 +99,7 @@ struct TraceArgs {
   int geo_mmax;
   const double* kap;     // kappa ds (rates.cu)
   const double* kappa;
+  const double* ikappa;  // 1/kappa
   int kap_mmax;
   TabDev tab;
   double tau_lim;
@@ -122,8 +125,8 @@ struct TraceArgs {
   const int* rtab_slot;   // R^2 limit -> slot, for 0..rtab_max_r2
   int rtab_max_r2;        // -1: no tables
   const int4* rtab_lay;   // per blob: offset, bytes, cells, half-width of the layer
-  const unsigned char* ftab;  // face tables (rates.cu) of the limits up to kFaceHcap
-  const int4* ftab_lay;       // the same for them, at the same entries
+  const unsigned char* ftab;  // face tables, up to a limit's first layer wider than kFaceHcap
+  const int4* ftab_lay;       // the same for them, at the same entries (0 bytes: none)
   // Interior row tables of the same (R^2 limit, m) layers, for faces traced
   // whole (see k_interior_tables): blob of layer m at itab + itab_off[same index].
   const unsigned char* itab;
@@ -205,6 +208,7 @@ struct Grid {
   unsigned char* ftab = nullptr;
   int4* ftab_lay = nullptr;
   int64_t ftab_bytes = 0;
+  int face_stack = 0;  // most cells of a face's layers up to its first wider than kBwdFaceHcap
   int rtab_max_r2 = -1;
   int rtab_mcap = 0;
   int64_t rtab_bytes = 0;
@@ -217,7 +221,7 @@ struct Grid {
   GeoEntry* geo = nullptr;
   GeoRow* georow = nullptr;
   int geo_mmax = 0;
-  double* kap = nullptr;  // kappa ds, then kappa, of the layers up to kap_mmax
+  double* kap = nullptr;  // kappa ds, then kappa, then 1/kappa, up to layer kap_mmax
   int kap_mmax = 0;
 
   // scratch
@@ -242,6 +246,8 @@ struct Grid {
   size_t bwd_stack_bytes = 0;
   double* dq_merged = nullptr;   // adjoint: dL/dlog Ndot per merged source
   int dq_cap = 0;
+  int* bwd_redo = nullptr;       // adjoint: quadrant items that whole faces left over
+  size_t bwd_redo_cap = 0;
   int bwd_exit = 1;              // adjoint: stop each item's recompute at its first opaque layer
   int interp_mode = 0;           // interpolation weights (rt_set_interpolation)
   double tau_w0 = 0.6;
@@ -334,10 +340,20 @@ cudaError_t launch_one_minus(const double* x, double* y, int64_t n, const int* s
                              cudaStream_t s);
 size_t face_stack_cap(int r2, int nmax);
 size_t bwd_smem_bytes(int hcap, int lcap);
-int bwd_max_grid(size_t smem, int block);
-cudaError_t launch_trace_bwd(Grid& g, const TraceArgs& t, const double* w, double* dlogn,
-                             double* dndot_merged, double2* stack, size_t stack_cap, int lcap,
-                             int grid, size_t smem, int block, bool exit);
+int bwd_max_grid(size_t smem, int block, int wpb = 0);
+size_t bwd_face_smem_bytes(int hcap);  // per warp
+// One launch of the adjoint (adjoint.cu): block 128 CTAs, 32 warps, 4 whole faces.
+struct BwdLaunch {
+  int block = 0, grid = 0, wpb = 0, lcap = 0;
+  size_t smem = 0, stack_cap = 0;
+  bool exit = true;
+  int* redo = nullptr;
+  int* redo_n = nullptr;
+  int redo_cap = 0, split_src = 0;
+  const int* n_dev = nullptr;
+};
+cudaError_t launch_trace_bwd(Grid& g, const TraceArgs& t, const BwdLaunch& L, const double* w,
+                             double* dlogn, double* dndot_merged, double2* stack);
 cudaError_t launch_dndot_inputs(Grid& g, const double* dmerged, double* out);
 cudaError_t launch_conv_check(const int64_t* unconv, int64_t limit, int* flag, cudaStream_t s);
 

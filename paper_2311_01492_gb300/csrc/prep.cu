@@ -200,7 +200,8 @@ __global__ void k_geometry(GeoEntry* __restrict__ geo, int mmax) {
 
 // Row-major entry (m, a1, a2) with the same correctly rounded expressions.
 __global__ void k_geometry_rows(GeoRow* __restrict__ geo, double* __restrict__ kap,
-                                double* __restrict__ kappa, const double2* __restrict__ binom, int mmax) {
+                                double* __restrict__ kappa, double* __restrict__ ikappa,
+                                const double2* __restrict__ binom, int mmax) {
   const int m = blockIdx.x + 1;
   if (m > mmax) return;
   const int cnt = (m + 1) * (m + 1);
@@ -224,19 +225,21 @@ __global__ void k_geometry_rows(GeoRow* __restrict__ geo, double* __restrict__ k
       const double2 k = kappa_dd(binom, m, a1, a2);
       kap[georow_index(m, a1, a2)] = fma(k.x, e.ds, k.y * e.ds);
       kappa[georow_index(m, a1, a2)] = k.x;
+      const double q = 1.0 / k.x;  // 1/kappa: one Newton step on the two-part kappa
+      ikappa[georow_index(m, a1, a2)] = q + q * (fma(-q, k.x, 1.0) - q * k.y);
     }
   }
 }
 
 // k = min(mmax, kKapMax): binom is scratch of (k + 1)(k + 2)/2 double2, kap holds
-// georow_count(k) values of kappa ds and then as many of kappa
+// georow_count(k) values of kappa ds, then as many of kappa, then of 1/kappa
 cudaError_t launch_geometry(GeoEntry* geo, GeoRow* georow, double* kap, double2* binom, int mmax,
                             cudaStream_t s) {
   if (mmax < 1) return cudaSuccess;
   k_binomials<<<std::min(mmax, kKapMax) + 1, 64, 0, s>>>(binom, std::min(mmax, kKapMax));
   count_launch();
-  k_geometry_rows<<<mmax, 256, 0, s>>>(georow, kap, kap + georow_count(std::min(mmax, kKapMax)), binom,
-                                       mmax);
+  const int64_t nk = georow_count(std::min(mmax, kKapMax));
+  k_geometry_rows<<<mmax, 256, 0, s>>>(georow, kap, kap + nk, kap + 2 * nk, binom, mmax);
   count_launch();
   k_geometry<<<mmax, 256, 0, s>>>(geo, mmax);
   count_launch();
@@ -599,39 +602,43 @@ __global__ void k_interior_tables(const int* __restrict__ ent_r2, const int* __r
 }
 
 // Cells of layer m of a whole face as signed offsets (t1, t2), two bytes each, in the
-// order that the in-place update of rates.cu needs, last first: quadrant positions (a1,
-// a2) by descending rows a1 and descending a2 (row a1 holds a2 = 0..min(H, isqrt(r2 - m^2 -
-// a1^2))), the distinct sign images of a position together.
-__global__ void k_face_tables(const int* __restrict__ ent_r2, const int* __restrict__ ent_m,
-                              const int4* __restrict__ lay, unsigned char* __restrict__ ftab,
-                              int nent) {
-  const int e = blockIdx.x;
-  if (e >= nent || lay[e].y == 0) return;
-  const int m = ent_m[e];
-  const int rem = ent_r2[e] - m * m;
+// order that the in-place update of rates.cu needs, last first: the cells off the axes by
+// quadrant position (a1, a2), descending rows a1 = H..1 and descending a2 (row a1 holds
+// a2 up to min(H, isqrt(r2 - m^2 - a1^2))), the four sign images of a position together
+// (they read axis slots, never the other way round); then the axes from a = H inwards,
+// (0, a) (0, -a) (a, 0) (-a, 0); the centre is entry 0.  job: (r2, m, offset, cells).
+__global__ void k_face_tables(const int4* __restrict__ job, unsigned char* __restrict__ ftab) {
+  const int4 q = job[blockIdx.x];
+  const int m = q.y;
+  const int rem = q.x - m * m;
   const int H = min(isqrt_dev(rem), m);
-  char2* out = reinterpret_cast<char2*>(ftab + lay[e].x);
-  __shared__ int at[kFaceHcap + 1];  // first entry of row a1
+  char2* out = reinterpret_cast<char2*>(ftab + q.z);
+  __shared__ int at[kFaceHcap + 2];  // positions off the axes in rows below a1
   if (threadIdx.x == 0) {
     int run = 0;
-    for (int a1 = H; a1 >= 0; --a1) {
+    for (int a1 = 1; a1 <= H; ++a1) {
       at[a1] = run;
-      run += (a1 ? 2 : 1) * (2 * min(H, isqrt_dev(rem - a1 * a1)) + 1);
+      run += min(H, isqrt_dev(rem - a1 * a1));
     }
+    out[0] = make_char2(0, 0);
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < (H + 1) * (H + 1); t += blockDim.x) {
-    const int a1 = t / (H + 1), a2 = t - a1 * (H + 1);
-    const int len = min(H, isqrt_dev(rem - a1 * a1));
-    if (a2 > len) continue;
-    const int n1 = a1 ? 2 : 1, n2 = a2 ? 2 : 1;
-    // (the cells are taken from the table's end)
-    char2* o = out + lay[e].z - 1 - (at[a1] + (len - a2) * 2 * n1);
-    for (int k = 0; k < n1 * n2; ++k)
-      o[-k] = make_char2((signed char)(k % n1 ? -a1 : a1), (signed char)(k / n1 ? -a2 : a2));
+  for (int a = 1 + threadIdx.x; a <= H; a += blockDim.x) {
+    char2* o = out + 4 * a;
+    o[0] = make_char2(0, (signed char)a);
+    o[-1] = make_char2(0, (signed char)-a);
+    o[-2] = make_char2((signed char)a, 0);
+    o[-3] = make_char2((signed char)-a, 0);
   }
-  for (int t = threadIdx.x; t < lay[e].y / 2 - lay[e].z; t += blockDim.x)  // the padding
-    out[lay[e].z + t] = make_char2(0, 0);
+  for (int t = threadIdx.x; t < H * H; t += blockDim.x) {
+    const int a1 = 1 + t / H, a2 = 1 + t % H;
+    if (a2 > min(H, isqrt_dev(rem - a1 * a1))) continue;
+    char2* o = out + 4 * H + 1 + 4 * (at[a1] + a2 - 1);
+    for (int k = 0; k < 4; ++k)
+      o[k] = make_char2((signed char)(k & 1 ? -a1 : a1), (signed char)(k & 2 ? -a2 : a2));
+  }
+  const int pad = ((2 * q.w + 15) & ~15) / 2 - q.w;
+  if (threadIdx.x < pad) out[q.w + threadIdx.x] = make_char2(0, 0);
 }
 
 void free_row_tables(Grid& g) {
@@ -665,9 +672,11 @@ rt_status ensure_row_tables(Grid& g) {
     g.rtab_mcap = mcap;
     return RT_OK;
   }
-  std::vector<int4> lay, flay;
+  std::vector<int4> lay, flay, jobs;
+  std::vector<int> square_at(kFaceHcap + 1, -1);
   std::vector<int> ent_r2, ent_m, off, ioff, first(r2s.size()), hcap(r2s.size());
   int64_t cur = 0, icur = 0, fcur = 0;
+  int face_stack = 0;
   for (size_t i = 0; i < r2s.size(); ++i) {
     const int v = r2s[i];
     const int L = std::min(isqrt_host(v), mcap);
@@ -698,15 +707,30 @@ rt_status ensure_row_tables(Grid& g) {
       }
     }
     hcap[i] = hc;
-    for (int m = 1; m <= L; ++m) {  // face tables of the narrow limits
-      if (hc > kFaceHcap) {
+    // face tables up to the limit's first layer wider than kFaceHcap; layers that are
+    // whole squares share one table
+    bool wide = false, bwd_fits = true;
+    int stack = 0;
+    for (int m = 1; m <= L; ++m) {
+      const int4 q = lay[first[i] + m - 1];
+      wide = wide || q.w > kFaceHcap;
+      if (wide) {
         flay.push_back(make_int4(0, 0, 0, 0));
         continue;
       }
-      const int4 q = lay[first[i] + m - 1];
       // four images of every position, less those that coincide on the two axes
       const int n = 4 * q.z - 4 * (q.w + 1) + 1;
       const int bytes = (2 * n + 15) & ~15;
+      bwd_fits = bwd_fits && q.w <= kBwdFaceHcap;
+      if (bwd_fits) stack += n;
+      face_stack = std::max(face_stack, stack);
+      const bool square = q.z == (m + 1) * (m + 1);
+      if (square && square_at[m] >= 0) {
+        flay.push_back(make_int4(square_at[m], bytes, n, q.w));
+        continue;
+      }
+      if (square) square_at[m] = (int)fcur;
+      jobs.push_back(make_int4(v, m, (int)fcur, n));
       flay.push_back(make_int4((int)fcur, bytes, n, q.w));
       fcur += bytes;
     }
@@ -718,6 +742,7 @@ rt_status ensure_row_tables(Grid& g) {
   std::vector<int> slot(maxv + 1, -1);
   for (size_t i = 0; i < r2s.size(); ++i) slot[r2s[i]] = (int)i;
   int *d_r2 = nullptr, *d_m = nullptr;
+  int4* d_jobs = nullptr;
   cudaStream_t s = g.stream;
 #undef CK
 #define CK(x)                                   \
@@ -744,6 +769,8 @@ rt_status ensure_row_tables(Grid& g) {
   CK(cudaMemcpyAsync(g.itab_off, ioff.data(), ioff.size() * sizeof(int), cudaMemcpyHostToDevice, s));
   CK(dev_malloc(&d_r2, std::max(nent, 1) * sizeof(int)));
   CK(dev_malloc(&d_m, std::max(nent, 1) * sizeof(int)));
+  CK(dev_malloc(&d_jobs, std::max<size_t>(jobs.size(), 1) * sizeof(int4)));
+  CK(cudaMemcpyAsync(d_jobs, jobs.data(), jobs.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(g.rtab_off, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(g.rtab_first, first.data(), first.size() * sizeof(int),
                      cudaMemcpyHostToDevice, s));
@@ -758,19 +785,19 @@ rt_status ensure_row_tables(Grid& g) {
     k_interior_tables<<<nent, 64, 0, s>>>(d_r2, d_m, g.itab_off, g.itab, nent);
     count_launch();
     CK(cudaGetLastError());
-    if (fcur > 0) {
-      k_face_tables<<<nent, 64, 0, s>>>(d_r2, d_m, g.ftab_lay, g.ftab, nent);
-      count_launch();
-      CK(cudaGetLastError());
-    }
+    k_face_tables<<<(int)jobs.size(), 64, 0, s>>>(d_jobs, g.ftab);
+    count_launch();
+    CK(cudaGetLastError());
   }
   CK(cudaStreamSynchronize(s));  // host vectors go out of scope
   dev_free(d_r2);
   dev_free(d_m);
+  dev_free(d_jobs);
   g.rtab_max_r2 = maxv;
   g.rtab_bytes = cur;
   g.itab_bytes = icur;
   g.ftab_bytes = fcur;
+  g.face_stack = face_stack;
   g.rtab_r2s = r2s;
   g.rtab_mcap = mcap;
   return RT_OK;
@@ -778,6 +805,7 @@ fail:
   cudaStreamSynchronize(s);
   dev_free(d_r2);
   dev_free(d_m);
+  dev_free(d_jobs);
   free_row_tables(g);
   return st;
 #undef CK
