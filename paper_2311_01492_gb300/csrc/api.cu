@@ -89,7 +89,7 @@ static void free_grid(Grid* g) {
   dev_free(g->dtau); dev_free(g->dtauT); dev_free(g->invn);
   free_sources(*g);
   dev_free(g->geo); dev_free(g->georow); dev_free(g->kap); dev_free(g->queue); dev_free(g->err);
-  dev_free(g->cube); dev_free(g->unconv); dev_free(g->xbuf); dev_free(g->xavg);
+  dev_free(g->cube); dev_free(g->od_scratch); dev_free(g->unconv); dev_free(g->xbuf); dev_free(g->xavg);
   dev_free(g->xavg2); dev_free(g->xhi_int); dev_free(g->flags); dev_free(g->counters);
   dev_free(g->bwd_stack); dev_free(g->dq_merged); dev_free(g->bwd_redo);
   free_row_tables(*g);
@@ -123,7 +123,7 @@ static rt_status ensure_geometry(Grid& g, int mmax) {
   double* kap = nullptr;
   double2* binom = nullptr;
   cudaError_t e = dev_malloc(&georow, georow_count(mmax) * sizeof(GeoRow));
-  if (e == cudaSuccess) e = dev_malloc(&kap, 3 * georow_count(kmax) * sizeof(double));
+  if (e == cudaSuccess) e = dev_malloc(&kap, 4 * georow_count(kmax) * sizeof(double));
   if (e == cudaSuccess) e = dev_malloc(&binom, (size_t)(kmax + 1) * (kmax + 2) / 2 * sizeof(double2));
   if (e == cudaSuccess) e = launch_geometry(geo, georow, kap, binom, mmax, g.stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(g.stream);  // binom is still read
@@ -145,12 +145,10 @@ static rt_status ensure_geometry(Grid& g, int mmax) {
   return RT_OK;
 }
 
-// Largest layer half-width min(m, floor(sqrt(r2 - m^2))) over the layers of a face.
+// Largest layer half-width min(m, floor(sqrt(r2 - m^2))) over the layers of a face (at
+// least 1): m grows up to sqrt(r2 / 2), beyond which the square root is the smaller.
 static int face_hcap(int r2, int nmax) {
-  int h = 1;
-  const int L = std::min(isqrt_h(r2), nmax / 2 + 1);
-  for (int m = 1; m <= L; ++m) h = std::max(h, std::min(m, isqrt_h((int64_t)r2 - (int64_t)m * m)));
-  return h;
+  return std::max(1, std::min({isqrt_h(r2), nmax / 2 + 1, isqrt_h(r2 / 2)}));
 }
 
 static TraceArgs base_args(Grid& g) {
@@ -185,6 +183,7 @@ static TraceArgs base_args(Grid& g) {
   a.kap_mmax = g.kap_mmax;
   a.kappa = g.kap ? g.kap + georow_count(g.kap_mmax) : nullptr;
   a.ikappa = g.kap ? g.kap + 2 * georow_count(g.kap_mmax) : nullptr;
+  a.dsik = g.kap ? g.kap + 3 * georow_count(g.kap_mmax) : nullptr;
   a.tab.g = g.gtab;
   a.tab.h = g.htab;
   a.tab.kind = g.tab_kind;
@@ -256,9 +255,6 @@ static rt_status ensure_cube(Grid& g, int nsrc, int* out_grid, int* out_E) {
   return RT_OK;
 }
 
-// Whether the batched rates go to rates.cu (its precompute: zeros for the thick terms).
-static bool takes_rates_kernels(const Grid& g) { return g.interp_mode == RT_INTERP_GEOMETRIC; }
-
 // First source (LPT order) whose layers fit half-width hlim; ns: none.
 static int first_fitting(const Grid& g, const int* r2s, int ns, int hlim) {
   if (hlim <= 0) return ns;
@@ -306,8 +302,12 @@ struct RatesPlan {
 // everything (64^3, 10 sources of R = 20: 0.048 against 0.057 ms; 128^3, 40 of R = 40:
 // 0.123 / 0.187).  With at most two items per SM they are the kAhead ones; with up to
 // four, CTAs of 256 pay for wide layers (200^3, 20 sources of R = 45: 0.146 / 0.177;
-// 128^3, 40 of R = 40, six items per SM: 0.156 / 0.128).
-static RatesPlan rates_plan(const Grid& g, const int* r2s, int ns) {
+// 128^3, 40 of R = 40, six items per SM: 0.156 / 0.128).  With the early exit an item
+// ends after a few layers and a wide one's latency counts: in a catalogue whose widest
+// quadrant takes a tenth of the whole, CTAs from half-width 20 on (128^3, early exit, CTA /
+// one quadrant, ms: 500 sources of R = 30 0.42 / 0.57 or 0.095 / 0.150 by cell size; 100
+// of R = 40 0.115 / 0.236; but 500 of R = 12 0.099 / 0.083).
+static RatesPlan rates_plan(const Grid& g, const int* r2s, int ns, bool exit) {
   RatesPlan p;
   p.mode[0] = g.block_big;
   p.cut[4] = ns;
@@ -328,7 +328,7 @@ static RatesPlan rates_plan(const Grid& g, const int* r2s, int ns) {
     p.cut[1] = p.cut[2] = p.cut[3] = ns;
     return p;
   }
-  const int lim[4] = {0, 38, 23, g.ftab ? 16 : 0};
+  const int lim[4] = {0, exit && longest_part(g, 24) > 0.1 ? 19 : 38, 23, g.ftab ? 16 : 0};
   for (int k = 1; k < 4; ++k) p.cut[k] = std::max(p.cut[k - 1], first_fitting(g, r2s, ns, lim[k]));
   for (int k = 3; k > 1; --k) {
     const double items = 24.0 / p.mode[k] * (p.cut[k + 1] - p.cut[k]);
@@ -337,46 +337,76 @@ static RatesPlan rates_plan(const Grid& g, const int* r2s, int ns) {
   return p;
 }
 
-static rt_status run_rates(Grid& g, const TraceArgs& a, const int* items, int ns) {
+// Whether the batched rates go to rates.cu (its precompute: zeros for the thick terms).
+// With optical-depth-modulated weights only its warps do; what needs CTAs takes trace.cu.
+static bool takes_rates_kernels(const Grid& g, bool exit) {
+  if (g.interp_mode == RT_INTERP_GEOMETRIC) return true;
+  return g.nsrc > 0 && g.od_scratch && rates_plan(g, g.r2_sorted_h.data(), g.nsrc, exit).cut[1] == 0;
+}
+
+struct RatesLaunch {
+  int mode, hcap, begin, end, grid, wpb;  // items [begin, end)
+  size_t smem;
+};
+static rt_status rates_launches(const Grid& g, bool exit, std::vector<RatesLaunch>& out) {
   const int* r2s = g.r2_sorted_h.data();
-  const RatesPlan plan = rates_plan(g, r2s, ns);
-  const int *mode = plan.mode, *cut = plan.cut;
-  TRY(cudaMemsetAsync(g.queue, 0, 4 * sizeof(int), g.stream));
+  const RatesPlan plan = rates_plan(g, r2s, g.nsrc, exit);
+  const bool od = g.interp_mode == RT_INTERP_OPTICAL_DEPTH;
   for (int k = 0; k < 4; ++k) {
-    if (cut[k + 1] <= cut[k]) continue;
-    TraceArgs b = a;
-    b.items = items;
-    b.hcap = face_hcap(r2s[cut[k]], g.nmax);
-    const int per = k == 0 ? 24 : 24 / mode[k];
-    b.item_begin = per * cut[k];
-    b.n_items = per * cut[k + 1];
-    b.queue = g.queue + k;
-    const size_t smem = rates_smem_bytes(b.hcap, mode[k]);
-    if (smem > 227 * 1024)
+    if (plan.cut[k + 1] <= plan.cut[k]) continue;
+    RatesLaunch L;
+    L.mode = plan.mode[k];
+    L.hcap = face_hcap(r2s[plan.cut[k]], g.nmax);
+    const int per = k == 0 ? 24 : 24 / L.mode;
+    L.begin = per * plan.cut[k];
+    L.end = per * plan.cut[k + 1];
+    L.smem = rates_smem_bytes(L.hcap, L.mode);
+    if (L.smem > 227 * 1024)
       return fail(RT_ERR_INVALID, "rt_raytrace: radius too large for the batched schedule's "
                                   "shared-memory layers; use RT_SCHED_PLAIN");
-    int wpb = 1, maxg = 0;
+    L.wpb = 1;
+    int maxg = 0;
     if (k == 0) {
-      maxg = rates_max_grid(mode[k], smem, 1, a.early_exit != 0);
+      maxg = rates_max_grid(L.mode, L.smem, 1, exit, od);
     } else {
       // CTAs of 1..8 warps, whichever keeps the most warps resident (a warp's shared
       // memory grows with its layer capacity, and every CTA also reserves some; ties
       // go to the larger CTA)
       for (int cand = 8; cand >= 1; --cand) {
-        const int mg = rates_max_grid(mode[k], smem * cand, cand, a.early_exit != 0);
-        if (mg * cand > maxg * wpb) {
+        const int mg = rates_max_grid(L.mode, L.smem * cand, cand, exit, od);
+        if (mg * cand > maxg * L.wpb) {
           maxg = mg;
-          wpb = cand;
+          L.wpb = cand;
         }
       }
     }
     if (maxg <= 0) return fail(RT_ERR_CUDA, "rt_raytrace: no occupancy for a rate kernel");
-    const int nitem = b.n_items - b.item_begin;
-    const int grid = mode[k] & kAhead ? nitem : std::max(1, std::min((nitem + wpb - 1) / wpb, maxg));
-    TRY(launch_rates(g, b, mode[k], grid, smem * wpb, wpb));
+    const int n = L.end - L.begin;
+    L.grid = L.mode & kAhead ? n : std::max(1, std::min((n + L.wpb - 1) / L.wpb, maxg));
+    L.smem *= L.wpb;
+    out.push_back(L);
+  }
+  return RT_OK;
+}
+
+static rt_status run_rates(Grid& g, const TraceArgs& a, const int* items) {
+  std::vector<RatesLaunch> ls;
+  rt_status st = rates_launches(g, a.early_exit != 0, ls);
+  if (st != RT_OK) return st;
+  TRY(cudaMemsetAsync(g.queue, 0, 4 * sizeof(int), g.stream));
+  for (size_t k = 0; k < ls.size(); ++k) {
+    const RatesLaunch& L = ls[k];
+    TraceArgs b = a;
+    b.items = items;
+    b.hcap = L.hcap;
+    b.item_begin = L.begin;
+    b.n_items = L.end;
+    b.queue = g.queue + k;
+    b.scratch = g.od_scratch;
+    TRY(launch_rates(g, b, L.mode, L.grid, L.smem, L.wpb));
     if (++g.stats.launches == 1) {
-      g.stats.block = k == 0 ? mode[k] & ~kAhead : 32 * wpb;
-      g.stats.grid = grid;
+      g.stats.block = L.mode <= 4 ? 32 * L.wpb : L.mode & ~kAhead;
+      g.stats.grid = L.grid;
     }
   }
   return RT_OK;
@@ -397,7 +427,7 @@ static rt_status run_trace(Grid& g, double* gamma, double* coldens, const int* i
   g.stats.launches = 0;
   TRY(cudaMemsetAsync(g.counters, 0, sizeof(unsigned long long), g.stream));
   const bool od = a.interp_mode == RT_INTERP_OPTICAL_DEPTH;
-  const bool rates = gamma && takes_rates_kernels(g);
+  const bool rates = gamma && takes_rates_kernels(g, early_exit);
   if (schedule != RT_SCHED_PLAIN && g.nmax > 1290)
     return fail(RT_ERR_INVALID, "rt_raytrace: the batched schedule needs boxes of at most "
                                 "1290^3 cells (32-bit offsets); use RT_SCHED_PLAIN");
@@ -417,7 +447,7 @@ static rt_status run_trace(Grid& g, double* gamma, double* coldens, const int* i
     g.stats.launches = 1;
     g.stats.items = nsrc_plain;
   } else if (rates) {
-    rt_status rs = run_rates(g, a, items, n_items / 24);
+    rt_status rs = run_rates(g, a, items);
     if (rs != RT_OK) return rs;
     TRY(launch_add_thick(g, gamma, skip));
     g.stats.items = n_items;
@@ -710,8 +740,9 @@ rt_status rt_raytrace(rt_grid_t h, double* d_gamma, int schedule) {
   if (st != RT_OK) return st;
   if (schedule == RT_SCHED_AUTO) schedule = g.auto_plain ? RT_SCHED_PLAIN : RT_SCHED_BATCHED;
   TRY(cudaEventRecord(g.ev[0], g.stream));
-  TRY(launch_precompute(g, schedule != RT_SCHED_PLAIN && takes_rates_kernels(g) ? PRE_THICK : PRE_INVN,
-                        d_gamma));
+  const bool rates = schedule != RT_SCHED_PLAIN &&
+                     takes_rates_kernels(g, schedule == RT_SCHED_BATCHED_EXIT);
+  TRY(launch_precompute(g, rates ? PRE_THICK : PRE_INVN, d_gamma));
   TRY(cudaEventRecord(g.ev[1], g.stream));
   if (g.nsrc > 0) {
     if (schedule == RT_SCHED_PLAIN)
@@ -739,7 +770,7 @@ rt_status rt_raytrace_source_coldens(rt_grid_t h, int src, double* d_coldens, in
   if (st != RT_OK) return st;
   TRY(launch_precompute(g, PRE_DTAU, d_coldens));
   const int hmax = face_hcap(g.max_r2, g.nmax);
-  if (schedule != RT_SCHED_PLAIN && takes_rates_kernels(g) && g.nmax <= 1290 &&
+  if (schedule != RT_SCHED_PLAIN && g.interp_mode == RT_INTERP_GEOMETRIC && g.nmax <= 1290 &&
       rates_smem_bytes(hmax, few_items_block(hmax)) <= 227 * 1024) {
     // 24 CTAs, their source looked up on the device, with room for the widest one:
     // nothing is asked back
@@ -873,7 +904,7 @@ rt_status rt_iterate(rt_grid_t h, double* d_x, double dt_s, double alpha_H, doub
     double* xin = (k % 2 == 0) ? g.xavg : g.xavg2;
     double* xout = (k % 2 == 0) ? g.xavg2 : g.xavg;
     TRY(launch_one_minus(xin, g.xhi_int, g.ncell, skip, g.stream));
-    TRY(launch_precompute(g, takes_rates_kernels(g) ? PRE_THICK : PRE_INVN, d_gamma, skip));
+    TRY(launch_precompute(g, takes_rates_kernels(g, false) ? PRE_THICK : PRE_INVN, d_gamma, skip));
     TRY(cudaMemsetAsync(g.unconv, 0, sizeof(int64_t), g.stream));
     if (g.nsrc > 0) {
       rt_status s2 = run_trace(g, d_gamma, nullptr, g.items, 24 * g.nsrc, RT_SCHED_BATCHED, g.nsrc, skip);
@@ -1099,6 +1130,19 @@ rt_status rt_set_interpolation(rt_grid_t h, int mode, double tau_weight_min) {
   if (!(tau_weight_min > 0.0) || !std::isfinite(tau_weight_min))
     return fail(RT_ERR_INVALID, "rt_set_interpolation: tau_weight_min must be finite and > 0");
   Grid& g = *reinterpret_cast<Grid*>(h);
+  if (mode == RT_INTERP_OPTICAL_DEPTH && !g.od_scratch) {
+    // Room for the reciprocals of every resident warp of rates.cu: no more than their layers
+    // take of the SMs' shared memory.  Here once, so that a trace allocates nothing and may
+    // be captured; without it (no memory, a capture under way) trace.cu, which needs none.
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(g.stream, &cap);
+    if (cap == cudaStreamCaptureStatusNone)
+      dev_malloc(&g.od_scratch, (size_t)sms * 228 * 1024);  // (null where it fails)
+    cudaGetLastError();
+  }
   g.interp_mode = mode;
   g.tau_w0 = tau_weight_min;
   ++g.epoch;
@@ -1202,7 +1246,7 @@ rt_status rt_autotune(rt_grid_t h, const char* cache_path, int* h_block, int* h_
   int bb = g.block_big, bh = g.hsmall, bf = 0;
   const bool was_explicit = g.explicit_schedule;
   g.explicit_schedule = false;
-  if (takes_rates_kernels(g)) timed(rule);
+  if (takes_rates_kernels(g, false)) timed(rule);
   g.explicit_schedule = true;
   g.hface = 0;
   for (int b : blocks)

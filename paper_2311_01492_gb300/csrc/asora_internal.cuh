@@ -100,12 +100,13 @@ struct TraceArgs {
   const double* kap;     // kappa ds (rates.cu)
   const double* kappa;
   const double* ikappa;  // 1/kappa
+  const double* dsik;    // ds/kappa
   int kap_mmax;
   TabDev tab;
   double tau_lim;
   double sigma0;
   int hcap;              // layer half-size capacity (faces) / cube half-size (shells)
-  double* scratch;       // per-CTA scratch (shell kernel)
+  double* scratch;       // per-CTA scratch (shell kernel), or per warp (rates.cu, mode 1)
   int* err;              // error flag (bit mask)
   const int* skip;       // if non-null and *skip != 0 the launch does nothing
   unsigned long long* rate_cells;  // number of rate evaluations (may be null)
@@ -221,13 +222,14 @@ struct Grid {
   GeoEntry* geo = nullptr;
   GeoRow* georow = nullptr;
   int geo_mmax = 0;
-  double* kap = nullptr;  // kappa ds, then kappa, then 1/kappa, up to layer kap_mmax
+  double* kap = nullptr;  // kappa ds, kappa, 1/kappa and ds/kappa, up to layer kap_mmax
   int kap_mmax = 0;
 
   // scratch
   int* queue = nullptr;
   int* err = nullptr;
   double* cube = nullptr;       // shell-kernel scratch
+  double* od_scratch = nullptr; // reciprocals of the batched rates with mode 1
   size_t cube_bytes = 0;
   int64_t* unconv = nullptr;    // iteration counters
   double* xbuf = nullptr;       // rt_iterate buffers
@@ -329,7 +331,7 @@ int shells_max_grid(int block);
 constexpr int kAhead = 1 << 12;
 cudaError_t launch_rates(Grid& g, const TraceArgs& a, int mode, int grid, size_t smem, int wpb);
 size_t rates_smem_bytes(int hcap, int mode);  // per CTA (warp modes: per warp)
-int rates_max_grid(int mode, size_t smem, int wpb, bool exit);
+int rates_max_grid(int mode, size_t smem, int wpb, bool exit, bool od);
 rt_status ingest_sources(Grid& g, int nsrc, const int32_t* d_pos, const int32_t* d_box,
                          const double* d_ndot, const double* d_radius);
 cudaError_t launch_chemistry(Grid& g, const double* gamma, const double* x0, const double* xavg_in,

@@ -201,7 +201,7 @@ __global__ void k_geometry(GeoEntry* __restrict__ geo, int mmax) {
 // Row-major entry (m, a1, a2) with the same correctly rounded expressions.
 __global__ void k_geometry_rows(GeoRow* __restrict__ geo, double* __restrict__ kap,
                                 double* __restrict__ kappa, double* __restrict__ ikappa,
-                                const double2* __restrict__ binom, int mmax) {
+                                double* __restrict__ dsik, const double2* __restrict__ binom, int mmax) {
   const int m = blockIdx.x + 1;
   if (m > mmax) return;
   const int cnt = (m + 1) * (m + 1);
@@ -226,20 +226,22 @@ __global__ void k_geometry_rows(GeoRow* __restrict__ geo, double* __restrict__ k
       kap[georow_index(m, a1, a2)] = fma(k.x, e.ds, k.y * e.ds);
       kappa[georow_index(m, a1, a2)] = k.x;
       const double q = 1.0 / k.x;  // 1/kappa: one Newton step on the two-part kappa
-      ikappa[georow_index(m, a1, a2)] = q + q * (fma(-q, k.x, 1.0) - q * k.y);
+      const double ik = q + q * (fma(-q, k.x, 1.0) - q * k.y);
+      ikappa[georow_index(m, a1, a2)] = ik;
+      dsik[georow_index(m, a1, a2)] = e.ds * ik;
     }
   }
 }
 
 // k = min(mmax, kKapMax): binom is scratch of (k + 1)(k + 2)/2 double2, kap holds
-// georow_count(k) values of kappa ds, then as many of kappa, then of 1/kappa
+// georow_count(k) values of kappa ds, then as many of kappa, 1/kappa and ds/kappa
 cudaError_t launch_geometry(GeoEntry* geo, GeoRow* georow, double* kap, double2* binom, int mmax,
                             cudaStream_t s) {
   if (mmax < 1) return cudaSuccess;
   k_binomials<<<std::min(mmax, kKapMax) + 1, 64, 0, s>>>(binom, std::min(mmax, kKapMax));
   count_launch();
   const int64_t nk = georow_count(std::min(mmax, kKapMax));
-  k_geometry_rows<<<mmax, 256, 0, s>>>(georow, kap, kap + nk, kap + 2 * nk, binom, mmax);
+  k_geometry_rows<<<mmax, 256, 0, s>>>(georow, kap, kap + nk, kap + 2 * nk, kap + 3 * nk, binom, mmax);
   count_launch();
   k_geometry<<<mmax, 256, 0, s>>>(geo, mmax);
   count_launch();

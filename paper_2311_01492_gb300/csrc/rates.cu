@@ -1,5 +1,5 @@
-// Batched trace of the photo-ionisation rates with the geometric weights
-// (RT_SCHED_BATCHED and its early exit; arXiv 2311.01492, Sec. 3.1-3.3).
+// Batched trace of the photo-ionisation rates (RT_SCHED_BATCHED and its early exit; arXiv
+// 2311.01492, Sec. 3.1-3.3), with the geometric weights unless said otherwise.
 //
 // The work items, their order and the geometry are those of trace.cu: a face of a
 // source is a square pyramid whose layer m depends only on layer m - 1, split into
@@ -76,6 +76,13 @@ __device__ __forceinline__ void source_rate(const TraceArgs& a, const Quad& Q, u
   if (dG != 0.0) atomicAdd(&(thin ? a.gamma : a.thick)[Q.scell], dG);
 }
 
+// The same with optical-depth-modulated weights; r: where s is in the reciprocals.
+__device__ __forceinline__ double interp_od(const TraceArgs& a, const Weights& w, const double* s,
+                                            const double* r, const int d1, const int d2) {
+  return od_interp_r(w.w12.x, w.w12.y, w.w34.x, w.w34.y, s[0], s[-d1], s[-d2], s[-d1 - d2], r[0],
+                     r[-d1], r[-d2], r[-d1 - d2], a.neg_zero);
+}
+
 // The rate of a cell of layer m >= 1 whose tau_in is within the tables (Eq. sugg; thin
 // limit Eq. gammalocal).  The thick terms are summed without their factor 1/n_HI,
 // which is the cell's own and is applied once to the sum (k_add_thick): one product
@@ -132,26 +139,32 @@ __device__ __forceinline__ int zero_count(int R2, int h) {
   return (min(h, isqrt_i(R2 >> 1)) + 2) * (h + 2);
 }
 
-// tau_out -> S for the cells of layer m (and whatever else lies in its square).
-template <int GS>
+// tau_out -> S (INV: P = kappa / tau_out) for the cells of layer m (and whatever else
+// lies in its square).
+template <int GS, bool INV = false>
 __device__ __forceinline__ void scale_layer(const TraceArgs& a, double* buf, const int W,
                                             const int m, const int h, const int gt) {
   const int H = min(m, h) + 1;
   const double* __restrict__ k = a.kappa + georow_index(m, 0, 0);
   for (int t = gt; t < H * H; t += GS) {
     const int a1 = t / H, a2 = t - a1 * H;
-    buf[(a1 + 1) * W + a2 + 1] *= __ldg(&k[a1 * (m + 1) + a2]);
+    double* p = &buf[(a1 + 1) * W + a2 + 1];
+    const double kappa = __ldg(&k[a1 * (m + 1) + a2]);
+    *p = INV ? kappa / *p : kappa * *p;
   }
 }
 
 // The same for a whole face.
+template <bool INV>
 __device__ __forceinline__ void scale_face(const TraceArgs& a, double* buf, const int W, const int m,
                                            const int h, const int lane) {
   const int H = min(m, h), S = 2 * H + 1;
   const double* __restrict__ k = a.kappa + georow_index(m, 0, 0);
   for (int t = lane; t < S * S; t += 32) {
     const int t1 = t / S - H, t2 = t % S - H;
-    buf[(t1 + h + 1) * W + t2 + h + 1] *= __ldg(&k[abs(t1) * (m + 1) + abs(t2)]);
+    double* p = &buf[(t1 + h + 1) * W + t2 + h + 1];
+    const double kappa = __ldg(&k[abs(t1) * (m + 1) + abs(t2)]);
+    *p = INV ? kappa / *p : kappa * *p;
   }
 }
 
@@ -167,9 +180,19 @@ __device__ __forceinline__ void scale_face(const TraceArgs& a, double* buf, cons
 // The indices and dtau of the next cells (of the next layer at a layer's
 // end) are loaded before a step is computed; a step of the scaled part takes two sets
 // of 32 cells, whose chains overlap.
-template <int MODE, bool EXIT>
+//
+// OD: optical-depth-modulated weights (od_interp_r).  Each slot's r = 1/max(tau_out,
+// tau_w0) lies beside the layer in a global scratch of the warp (rbuf; shared memory for
+// both would halve the resident warps, and this part is FP64-bound).  Once all is opaque,
+// and beyond tau_w0, every product r tau is one and the normalised sum is the weighted
+// harmonic mean: with P = kappa / tau_out,
+//   D = kappa / tau_in = P(a1,a2) + P(a1-1,a2) + P(a1,a2-1) + P(a1-1,a2-1)
+//   P = kappa / (kappa / D + dtau ds) = D / fma(dtau, D (ds / kappa), 1)
+// one division instead of two, and no weights.
+template <int MODE, bool EXIT, bool OD>
 __device__ __forceinline__ void rates_item_warp(const TraceArgs& a, const int item, const int lane,
-                                                unsigned char* __restrict__ sm, const int h,
+                                                unsigned char* __restrict__ sm,
+                                                double* __restrict__ rbuf, const int h,
                                                 unsigned& nrate) {
   constexpr unsigned FULL = 0xffffffffu;
   constexpr bool FACE = MODE == 4;
@@ -183,6 +206,8 @@ __device__ __forceinline__ void rates_item_warp(const TraceArgs& a, const int it
   double* buf = reinterpret_cast<double*>(sm + (FACE ? 0 : (lane / P) * rates_buf_bytes(h)));
   unsigned char* tab = sm + (FACE ? face_layer_bytes(h) : K * rates_buf_bytes(h));
   double* const org = FACE ? buf + (h + 1) * (W + 1) : buf + W + 1;  // slot of (0, 0)
+  double* const rorg =
+      OD ? rbuf + (FACE ? (h + 1) * (W + 1) : (lane / P) * (h + 2) * (h + 2) + W + 1) : nullptr;
   if (FACE) {
     const int hz = min(h, isqrt_i(Q.R2 >> 1));
     for (int t = (h - hz) * W + lane; t < (h + hz + 3) * W; t += 32) buf[t] = 0.0;
@@ -298,11 +323,13 @@ __device__ __forceinline__ void rates_item_warp(const TraceArgs& a, const int it
     double* sc = org + c.t1 * W + c.t2;
     double tin;
     if constexpr (FIRST) tin = Q.half_dts * w.ds;  // source centre to the layer's entry plane
+    else if constexpr (OD) tin = interp_od(a, w, sc, rorg + c.t1 * W + c.t2, d1_of(c), d2_of(c));
     else tin = interp(a, w, sc, d1_of(c), d2_of(c));
     const double tout = fma(c.dtp, w.ds, tin);
     __syncwarp();  // all reads before any write
     if (Tc - lq >= 0 && in_window(c)) {
       *sc = tout;
+      if (OD) rorg[c.t1 * W + c.t2] = od_recip(tout, a.tau_w0);
       opaque = opaque && bits_of(tout) >= a.exit_bits;
       if (bits_of(tin) < a.tab.tau_max_bits)
         deposit_rate<FACE>(a, Q, mc, c, gr, w.ds, tin, tout, nrate);
@@ -313,27 +340,30 @@ __device__ __forceinline__ void rates_item_warp(const TraceArgs& a, const int it
     opaque = true;
     return all;
   };
-  bool done = step(std::true_type());
-  while (T0 >= 0 && !done) done = step(std::false_type());
+  // (OD: the scaled form also needs every column beyond tau_w0)
+  const bool scalable = !OD || bits_of(a.tau_w0) <= a.exit_bits;
+  bool done = step(std::true_type()) && (EXIT || scalable);
+  while (T0 >= 0 && !done) done = step(std::false_type()) && (EXIT || scalable);
   if (EXIT || T0 < 0) {
     cp_async_wait_all();  // (a copy may be in flight)
     return;
   }
   // ---- no rates any more: the column densities in scaled form
-  if (FACE) scale_face(a, buf, W, m - 1, h, lane);
-  else scale_layer<P>(a, buf, W, m - 1, h, lq);
+  if (FACE) scale_face<OD>(a, buf, W, m - 1, h, lane);
+  else scale_layer<P, OD>(a, buf, W, m - 1, h, lq);
   __syncwarp();
+  const double* __restrict__ geo = OD ? a.dsik : a.kap;
   CellIn ne;
   auto prefetch = [&]() {
-    nc.kds = __ldg(&a.kap[fetch(nc, max(T0 - lq, 0))]);
-    if (T0 >= P) ne.kds = __ldg(&a.kap[fetch(ne, max(T0 - P - lq, 0))]);
+    nc.kds = __ldg(&geo[fetch(nc, max(T0 - lq, 0))]);
+    if (T0 >= P) ne.kds = __ldg(&geo[fetch(ne, max(T0 - P - lq, 0))]);
   };
-  auto column = [&](const CellIn& c, const double* s) {  // S of the cell at slot s
+  auto column = [&](const CellIn& c, const double* s) {  // S (P) of the cell at slot s
     const int d1 = d1_of(c), d2 = d2_of(c);
     const bool z1 = FACE && c.t1 == 0, z2 = FACE && c.t2 == 0;  // nothing beyond an axis
     const double v = bracket_sum(s[0], z1 ? buf[0] : s[-d1], z2 ? buf[0] : s[-d2],
                                  z1 || z2 ? buf[0] : s[-d1 - d2]);
-    return fma(c.dtp, c.kds, v);
+    return OD ? v / fma(c.dtp, v * c.kds, 1.0) : fma(c.dtp, c.kds, v);
   };
   prefetch();
   while (T0 >= 0) {
@@ -551,19 +581,31 @@ __global__ void __launch_bounds__(BLOCK, (AHEAD ? 512 : 1024) / BLOCK) k_rates_c
   if (WHAT != COLDENS) flush_rates(a, nrate);
 }
 
-template <int MODE, bool EXIT>
+// Doubles of one layer buffer of a warp (all its quadrants, or its face).
+__host__ __device__ inline size_t warp_slots(int h, int mode) {
+  return mode == 4 ? (size_t)(2 * h + 3) * (2 * h + 3) : (size_t)mode * (h + 2) * (h + 2);
+}
+
+template <int MODE, bool EXIT, bool OD>
 __global__ void __launch_bounds__(256, 2) k_rates_warp(TraceArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (a.skip && *a.skip) return;
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned char* my = smem_raw + (size_t)wid * rates_warp_bytes(a.hcap, MODE);
+  double* rbuf = nullptr;
+  if (OD) {  // finite values in every slot that a zero weight may read
+    const size_t n = warp_slots(a.hcap, MODE);
+    rbuf = a.scratch + ((size_t)blockIdx.x * (blockDim.x >> 5) + wid) * n;
+    for (size_t t = lane; t < n; t += 32) rbuf[t] = 0.0;
+    __syncwarp();
+  }
   unsigned nrate = 0;
   for (;;) {
     int it = 0;
     if (lane == 0) it = a.item_begin + atomicAdd(a.queue, 1);
     it = __shfl_sync(0xffffffffu, it, 0);
     if (it >= a.n_items) break;
-    rates_item_warp<MODE, EXIT>(a, a.items[it * MODE], lane, my, a.hcap, nrate);
+    rates_item_warp<MODE, EXIT, OD>(a, a.items[it * MODE], lane, my, rbuf, a.hcap, nrate);
     __syncwarp();
   }
   flush_rates(a, nrate);
@@ -571,39 +613,37 @@ __global__ void __launch_bounds__(256, 2) k_rates_warp(TraceArgs a) {
 
 // mode: quadrants per warp (1, 2), 4: a whole face per warp, or threads of a CTA (128,
 // 256; with kAhead 128, 256, 512)
-static const void* rates_kernel(int mode, int what) {
-#define ASORA_PICK(K, ...)                                                \
-  (what == RATES_EXIT ? (const void*)K<__VA_ARGS__ RATES_EXIT ASORA_REST> \
-                      : (const void*)K<__VA_ARGS__ RATES ASORA_REST>)
-#define ASORA_REST
+static const void* rates_kernel(int mode, int what, bool od) {
+  const bool exit = what == RATES_EXIT;
+#define ASORA_WARP(M)                                                                          \
+  (od ? exit ? (const void*)k_rates_warp<M, true, true> : (const void*)k_rates_warp<M, false, true> \
+      : exit ? (const void*)k_rates_warp<M, true, false>                                       \
+             : (const void*)k_rates_warp<M, false, false>)
+#define ASORA_CTA(B, AHEAD)                                      \
+  (od ? nullptr : exit ? (const void*)k_rates_cta<B, RATES_EXIT, AHEAD> \
+                       : (const void*)k_rates_cta<B, RATES, AHEAD>)
+#define ASORA_AHEAD(B) \
+  (what == COLDENS ? (const void*)k_rates_cta<B, COLDENS, true> : ASORA_CTA(B, true))
   switch (mode) {
-    case 1: return ASORA_PICK(k_rates_warp, 1, );
-    case 2: return ASORA_PICK(k_rates_warp, 2, );
-    case 4: return ASORA_PICK(k_rates_warp, 4, );
-#undef ASORA_REST
-#define ASORA_REST , false
-    case 128: return ASORA_PICK(k_rates_cta, 128, );
-    case 256: return ASORA_PICK(k_rates_cta, 256, );
-#undef ASORA_REST
-#define ASORA_REST , true
-    case 128 | kAhead:
-      return what == COLDENS ? (const void*)k_rates_cta<128, COLDENS, true>
-                             : ASORA_PICK(k_rates_cta, 128, );
-    case 256 | kAhead:
-      return what == COLDENS ? (const void*)k_rates_cta<256, COLDENS, true>
-                             : ASORA_PICK(k_rates_cta, 256, );
-    case 512 | kAhead:
-      return what == COLDENS ? (const void*)k_rates_cta<512, COLDENS, true>
-                             : ASORA_PICK(k_rates_cta, 512, );
+    case 1: return ASORA_WARP(1);
+    case 2: return ASORA_WARP(2);
+    case 4: return ASORA_WARP(4);
+    case 128: return ASORA_CTA(128, false);
+    case 256: return ASORA_CTA(256, false);
+    case 128 | kAhead: return ASORA_AHEAD(128);
+    case 256 | kAhead: return ASORA_AHEAD(256);
+    case 512 | kAhead: return ASORA_AHEAD(512);
     default: return nullptr;
   }
-#undef ASORA_REST
-#undef ASORA_PICK
+#undef ASORA_AHEAD
+#undef ASORA_CTA
+#undef ASORA_WARP
 }
 
 cudaError_t launch_rates(Grid& g, const TraceArgs& a, int mode, int grid, size_t smem, int wpb) {
   const void* fn =
-      rates_kernel(mode, a.coldens ? COLDENS : a.early_exit ? RATES_EXIT : RATES);
+      rates_kernel(mode, a.coldens ? COLDENS : a.early_exit ? RATES_EXIT : RATES,
+                   !a.coldens && a.interp_mode == RT_INTERP_OPTICAL_DEPTH);
   if (!fn) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -615,11 +655,11 @@ cudaError_t launch_rates(Grid& g, const TraceArgs& a, int mode, int grid, size_t
   return e;
 }
 
-int rates_max_grid(int mode, size_t smem, int wpb, bool exit) {
+int rates_max_grid(int mode, size_t smem, int wpb, bool exit, bool od) {
   int dev = 0, sms = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const void* fn = rates_kernel(mode, exit ? RATES_EXIT : RATES);
+  const void* fn = rates_kernel(mode, exit ? RATES_EXIT : RATES, od);
   if (!fn) return 0;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess)
