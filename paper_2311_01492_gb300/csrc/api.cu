@@ -284,10 +284,11 @@ static double longest_part(const Grid& g, int parts) {
 }
 
 // Launches of the batched rates: sources [cut[k], cut[k+1]) (LPT order) by CTAs of
-// mode[0] threads (k = 0) or by warps with one quadrant, two, or a whole face (k = 1..3).
+// mode[0] threads (k = 0) or by warps with one quadrant, two, or a whole face (k > 0).
 struct RatesPlan {
-  int mode[4] = {128, 1, 2, 4};
-  int cut[5] = {0, 0, 0, 0, 0};
+  static constexpr int kClasses = 5;
+  int mode[kClasses] = {128, 1, 1, 2, 4};
+  int cut[kClasses + 1] = {};
 };
 
 // With rt_set_schedule (or an autotuned choice): its thresholds.  Otherwise by rule.
@@ -295,7 +296,10 @@ struct RatesPlan {
 // / two / a face; 128^3): R = 12 (half-width 8), 4e4 sources 16.7 / 10.4 / 7.3 / 5.2;
 // R = 22 (15), 1e4: 7.4 / 4.7 / 4.0 / 3.7; R = 27 (19), 8e3: 7.7 / 5.1 / 4.7 / 5.8;
 // R = 33 (23), 5e3: 6.5 / 4.8 / 4.6 / -; R = 50 (35), 2e3: 5.8 / 5.3 / 7.0 / -; R = 60
-// (42), 1e3: 4.8 / 5.3 / - / -: hence the half-widths.  A launch pays for its last
+// (42), 1e3: 4.8 / 5.3 / - / -: hence the half-widths.  One quadrant
+// per warp is launched twice, as its warps' shared memory goes by the widest source: from
+// half-width 30 on 14 warps fit an SM, below 21 (250^3, 3e5 sources of R = 5..50: 143.4 /
+// 138.2 ms in four launches).  A launch pays for its last
 // wave, so where several classes would be launched a class of few items joins the finer
 // one before it (64^3, 1e3 sources of R = 5..50: one launch 0.52, three 0.87 ms), and
 // where one quadrant would take a warp longer than all work takes the GPU, CTAs trace
@@ -310,10 +314,12 @@ struct RatesPlan {
 static RatesPlan rates_plan(const Grid& g, const int* r2s, int ns, bool exit) {
   RatesPlan p;
   p.mode[0] = g.block_big;
-  p.cut[4] = ns;
+  constexpr int K = RatesPlan::kClasses;
+  p.cut[K] = ns;
   if (g.explicit_schedule) {
     p.cut[1] = first_fitting(g, r2s, ns, g.hsmall);
-    p.cut[2] = p.cut[3] = g.ftab ? std::max(p.cut[1], first_fitting(g, r2s, ns, g.hface)) : ns;
+    for (int k = 2; k < K; ++k)
+      p.cut[k] = g.ftab ? std::max(p.cut[1], first_fitting(g, r2s, ns, g.hface)) : ns;
     return p;
   }
   int dev = 0, sms = 0;
@@ -325,12 +331,12 @@ static RatesPlan rates_plan(const Grid& g, const int* r2s, int ns, bool exit) {
     const int h = face_hcap(r2s[0], g.nmax);
     if (24 * ns <= 2 * sms) p.mode[0] = few_items_block(h);
     else if (24 * ns <= 4 * sms && h >= 24) p.mode[0] = 256;
-    p.cut[1] = p.cut[2] = p.cut[3] = ns;
+    for (int k = 1; k < K; ++k) p.cut[k] = ns;
     return p;
   }
-  const int lim[4] = {0, exit && longest_part(g, 24) > 0.1 ? 19 : 38, 23, g.ftab ? 16 : 0};
-  for (int k = 1; k < 4; ++k) p.cut[k] = std::max(p.cut[k - 1], first_fitting(g, r2s, ns, lim[k]));
-  for (int k = 3; k > 1; --k) {
+  const int lim[K] = {0, exit && longest_part(g, 24) > 0.1 ? 19 : 38, 30, 23, g.ftab ? 16 : 0};
+  for (int k = 1; k < K; ++k) p.cut[k] = std::max(p.cut[k - 1], first_fitting(g, r2s, ns, lim[k]));
+  for (int k = K - 1; k > 1; --k) {
     const double items = 24.0 / p.mode[k] * (p.cut[k + 1] - p.cut[k]);
     if (items < (p.cut[k] > 0 ? 6 : 1.2) * warps) p.cut[k] = p.cut[k + 1];
   }
@@ -352,7 +358,7 @@ static rt_status rates_launches(const Grid& g, bool exit, std::vector<RatesLaunc
   const int* r2s = g.r2_sorted_h.data();
   const RatesPlan plan = rates_plan(g, r2s, g.nsrc, exit);
   const bool od = g.interp_mode == RT_INTERP_OPTICAL_DEPTH;
-  for (int k = 0; k < 4; ++k) {
+  for (int k = 0; k < RatesPlan::kClasses; ++k) {
     if (plan.cut[k + 1] <= plan.cut[k]) continue;
     RatesLaunch L;
     L.mode = plan.mode[k];
@@ -369,10 +375,10 @@ static rt_status rates_launches(const Grid& g, bool exit, std::vector<RatesLaunc
     if (k == 0) {
       maxg = rates_max_grid(L.mode, L.smem, 1, exit, od);
     } else {
-      // CTAs of 1..8 warps, whichever keeps the most warps resident (a warp's shared
-      // memory grows with its layer capacity, and every CTA also reserves some; ties
-      // go to the larger CTA)
-      for (int cand = 8; cand >= 1; --cand) {
+      // CTAs of as many warps as keeps the most resident (a warp's shared memory grows
+      // with its layer capacity, and every CTA also reserves some; ties go to the
+      // larger CTA)
+      for (int cand = rates_max_warps(L.mode, exit, od); cand >= 1; --cand) {
         const int mg = rates_max_grid(L.mode, L.smem * cand, cand, exit, od);
         if (mg * cand > maxg * L.wpb) {
           maxg = mg;
@@ -393,7 +399,7 @@ static rt_status run_rates(Grid& g, const TraceArgs& a, const int* items) {
   std::vector<RatesLaunch> ls;
   rt_status st = rates_launches(g, a.early_exit != 0, ls);
   if (st != RT_OK) return st;
-  TRY(cudaMemsetAsync(g.queue, 0, 4 * sizeof(int), g.stream));
+  TRY(cudaMemsetAsync(g.queue, 0, RatesPlan::kClasses * sizeof(int), g.stream));
   for (size_t k = 0; k < ls.size(); ++k) {
     const RatesLaunch& L = ls[k];
     TraceArgs b = a;

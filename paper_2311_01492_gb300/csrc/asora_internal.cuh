@@ -331,6 +331,7 @@ int shells_max_grid(int block);
 constexpr int kAhead = 1 << 12;
 cudaError_t launch_rates(Grid& g, const TraceArgs& a, int mode, int grid, size_t smem, int wpb);
 size_t rates_smem_bytes(int hcap, int mode);  // per CTA (warp modes: per warp)
+int rates_max_warps(int mode, bool exit, bool od);  // per CTA (modes 1, 2, 4)
 int rates_max_grid(int mode, size_t smem, int wpb, bool exit, bool od);
 rt_status ingest_sources(Grid& g, int nsrc, const int32_t* d_pos, const int32_t* d_box,
                          const double* d_ndot, const double* d_radius);

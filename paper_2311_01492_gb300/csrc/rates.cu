@@ -586,8 +586,22 @@ __host__ __device__ inline size_t warp_slots(int h, int mode) {
   return mode == 4 ? (size_t)(2 * h + 3) * (2 * h + 3) : (size_t)mode * (h + 2) * (h + 2);
 }
 
+// Threads of a CTA and CTAs per SM that the registers are cut for.  The scaled part waits
+// for loads and shared memory, so warps count: with 16 (127 registers), 20 (96) or 21 (90)
+// per SM a batched trace of 128^3 takes, in one quadrant per warp (half-width 23, 5e3
+// sources) 4.76 / 4.41 / 4.28 ms, in whole faces (11, 2e4) 3.02 / 2.76 / 2.65, in two
+// quadrants (15, 2e4; 90 registers spill) 4.28 / 4.02 / 4.82.  With optical-depth weights
+// 7.19 / 7.26 / 7.31, with rates everywhere 2.33 / 2.29 / 2.31: FP64-bound.
+__host__ __device__ constexpr int rates_warps(int mode, bool exit, bool od) {
+  return od ? 8 : mode == 2 || (mode == 4 && exit) ? 4 : 3;
+}
+__host__ __device__ constexpr int rates_ctas(int mode, bool exit, bool od) {
+  return od ? 2 : mode == 2 || (mode == 4 && exit) ? 5 : 7;
+}
+
 template <int MODE, bool EXIT, bool OD>
-__global__ void __launch_bounds__(256, 2) k_rates_warp(TraceArgs a) {
+__global__ void __launch_bounds__(32 * rates_warps(MODE, EXIT, OD), rates_ctas(MODE, EXIT, OD))
+k_rates_warp(TraceArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (a.skip && *a.skip) return;
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -654,6 +668,8 @@ cudaError_t launch_rates(Grid& g, const TraceArgs& a, int mode, int grid, size_t
   count_launch();
   return e;
 }
+
+int rates_max_warps(int mode, bool exit, bool od) { return rates_warps(mode, exit, od); }
 
 int rates_max_grid(int mode, size_t smem, int wpb, bool exit, bool od) {
   int dev = 0, sms = 0, per = 0;
