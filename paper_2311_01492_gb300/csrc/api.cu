@@ -299,7 +299,8 @@ struct RatesPlan {
 // (42), 1e3: 4.8 / 5.3 / - / -: hence the half-widths.  One quadrant
 // per warp is launched twice, as its warps' shared memory goes by the widest source: from
 // half-width 30 on 14 warps fit an SM, below 21 (250^3, 3e5 sources of R = 5..50: 143.4 /
-// 138.2 ms in four launches).  A launch pays for its last
+// 138.2 ms in four launches; 128^3, 1.6e4 7.26 / 7.21, with the early exit 1.18 / 1.28;
+// 64^3, 1e3 0.47 / 0.54: only where both parts are large).  A launch pays for its last
 // wave, so where several classes would be launched a class of few items joins the finer
 // one before it (64^3, 1e3 sources of R = 5..50: one launch 0.52, three 0.87 ms), and
 // where one quadrant would take a warp longer than all work takes the GPU, CTAs trace
@@ -337,7 +338,8 @@ static RatesPlan rates_plan(const Grid& g, const int* r2s, int ns, bool exit) {
   const int lim[K] = {0, exit && longest_part(g, 24) > 0.1 ? 19 : 38, 30, 23, g.ftab ? 16 : 0};
   for (int k = 1; k < K; ++k) p.cut[k] = std::max(p.cut[k - 1], first_fitting(g, r2s, ns, lim[k]));
   for (int k = K - 1; k > 1; --k) {
-    const double items = 24.0 / p.mode[k] * (p.cut[k + 1] - p.cut[k]);
+    double items = 24.0 / p.mode[k] * (p.cut[k + 1] - p.cut[k]);
+    if (k == 2) items = std::min(items, 24.0 * (p.cut[2] - p.cut[1])) / (exit ? 6 : 2);
     if (items < (p.cut[k] > 0 ? 6 : 1.2) * warps) p.cut[k] = p.cut[k + 1];
   }
   return p;
