@@ -9,6 +9,7 @@
 // given one times inv_a3 = a^-3 in an expanding background, an exact no-op for
 // a = 1).  Built with --fmad=false so the expressions round exactly as written.
 #include "asora_internal.cuh"
+#include "quick_div.cuh"
 
 namespace asora {
 
@@ -79,8 +80,8 @@ __global__ void k_chemistry(int64_t n, const double* __restrict__ nH, double inv
         xeq_last = diff;
         mean = fma(-y, q, 1.0);
       } else if (decays) {
-        const double xeq = num / rate;
-        xa_new = xeq + (xs - xeq) * (-expm1(-y) / y);
+        const double xeq = quick_div(num, rate);
+        xa_new = xeq + (xs - xeq) * quick_div(-expm1(-y), y);
         xeq_last = xeq;
         y_last = y;
       } else {

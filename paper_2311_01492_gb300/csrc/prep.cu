@@ -9,6 +9,7 @@
 #include <map>
 
 #include "asora_internal.cuh"
+#include "device_util.cuh"
 
 namespace asora {
 
@@ -73,7 +74,7 @@ __global__ void k_precompute(const BoxDev* __restrict__ boxes, const double* __r
         const double nh = nH[idx] * inv_a3, x = xHI[idx];
         const double d = (B.sig_cell * nh) * x;
         dtau[idx] = d;
-        if (WHAT == PRE_INVN) invn[idx] = 1.0 / (nh * x);
+        if (WHAT == PRE_INVN) invn[idx] = quick_recip(nh * x);
         if (WHAT == PRE_THICK) invn[idx] = 0.0;
         if (out) out[idx] = 0.0;
         tile[yy][tx] = d;
@@ -106,7 +107,7 @@ __global__ void k_tau_to_coldens(int64_t n, double sigma0, double* __restrict__ 
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
        t += (int64_t)gridDim.x * blockDim.x) {
     const double v = c[t];
-    if (v != 0.0) c[t] = v / sigma0;
+    if (bits_of(v)) c[t] = quick_div(v, sigma0);
   }
 }
 
@@ -117,7 +118,10 @@ cudaError_t launch_tau_to_coldens(Grid& g, double* coldens) {
   return cudaGetLastError();
 }
 
-// gamma += thick / n_HI (Eq. sugg's 1/n_HI, taken out of the sum over sources)
+// gamma += thick / n_HI (Eq. sugg's 1/n_HI, taken out of the sum over sources).  FP64 issue
+// binds while a cell takes more than three instructions (4 fields through memory: 74 us at
+// 250^3): 165 us, and 350 with a / b, 1/a^3 always applied and a test in FP64.
+template <bool SCALED>
 __global__ void k_add_thick(int64_t n, const double* __restrict__ nH, const double* __restrict__ xHI,
                             double inv_a3, const double* __restrict__ thick,
                             double* __restrict__ gamma, const int* __restrict__ skip) {
@@ -125,13 +129,14 @@ __global__ void k_add_thick(int64_t n, const double* __restrict__ nH, const doub
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n;
        c += (int64_t)gridDim.x * blockDim.x) {
     const double t = thick[c];
-    if (t != 0.0) gamma[c] += t / ((nH[c] * inv_a3) * xHI[c]);
+    if (bits_of(t)) gamma[c] += quick_div(t, (SCALED ? nH[c] * inv_a3 : nH[c]) * xHI[c]);
   }
 }
 
 cudaError_t launch_add_thick(Grid& g, double* gamma, const int* skip) {
   const int grid = (int)std::min<int64_t>((g.ncell + 255) / 256, 152 * 16);
-  k_add_thick<<<grid, 256, 0, g.stream>>>(g.ncell, g.nH, g.xHI, g.inv_a3, g.invn, gamma, skip);
+  auto* k = g.inv_a3 != 1.0 ? k_add_thick<true> : k_add_thick<false>;
+  k<<<grid, 256, 0, g.stream>>>(g.ncell, g.nH, g.xHI, g.inv_a3, g.invn, gamma, skip);
   count_launch();
   return cudaGetLastError();
 }

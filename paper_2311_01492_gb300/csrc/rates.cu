@@ -150,7 +150,7 @@ __device__ __forceinline__ void scale_layer(const TraceArgs& a, double* buf, con
     const int a1 = t / H, a2 = t - a1 * H;
     double* p = &buf[(a1 + 1) * W + a2 + 1];
     const double kappa = __ldg(&k[a1 * (m + 1) + a2]);
-    *p = INV ? kappa / *p : kappa * *p;
+    *p = INV ? quick_div(kappa, *p) : kappa * *p;
   }
 }
 
@@ -164,7 +164,7 @@ __device__ __forceinline__ void scale_face(const TraceArgs& a, double* buf, cons
     const int t1 = t / S - H, t2 = t % S - H;
     double* p = &buf[(t1 + h + 1) * W + t2 + h + 1];
     const double kappa = __ldg(&k[abs(t1) * (m + 1) + abs(t2)]);
-    *p = INV ? kappa / *p : kappa * *p;
+    *p = INV ? quick_div(kappa, *p) : kappa * *p;
   }
 }
 
@@ -363,7 +363,7 @@ __device__ __forceinline__ void rates_item_warp(const TraceArgs& a, const int it
     const bool z1 = FACE && c.t1 == 0, z2 = FACE && c.t2 == 0;  // nothing beyond an axis
     const double v = bracket_sum(s[0], z1 ? buf[0] : s[-d1], z2 ? buf[0] : s[-d2],
                                  z1 || z2 ? buf[0] : s[-d1 - d2]);
-    return OD ? v / fma(c.dtp, v * c.kds, 1.0) : fma(c.dtp, c.kds, v);
+    return OD ? quick_div(v, fma(c.dtp, v * c.kds, 1.0)) : fma(c.dtp, c.kds, v);
   };
   prefetch();
   while (T0 >= 0) {
