@@ -108,8 +108,6 @@ __device__ __forceinline__ double group_sum(double v, double* red, int gt) {
   return s;
 }
 
-__device__ __forceinline__ bool nonzero(double x) { return (bits_of(x) << 1) != 0; }
-
 // Direct terms of an owned cell with a rate and w != 0: adds w Gamma to qacc and returns
 // dL/dtau_in; lam (in: what arrives from the cell's users) becomes dL/dtau_out, ndir the
 // 1/n_HI term of dL/dlog n_HI.  In the thick form the two derivatives combine as the slope

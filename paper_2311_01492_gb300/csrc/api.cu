@@ -125,7 +125,7 @@ static rt_status ensure_geometry(Grid& g, int mmax) {
   cudaError_t e = dev_malloc(&georow, georow_count(mmax) * sizeof(GeoRow));
   if (e == cudaSuccess) e = dev_malloc(&kap, 4 * georow_count(kmax) * sizeof(double));
   if (e == cudaSuccess) e = dev_malloc(&binom, (size_t)(kmax + 1) * (kmax + 2) / 2 * sizeof(double2));
-  if (e == cudaSuccess) e = launch_geometry(geo, georow, kap, binom, mmax, g.stream);
+  if (e == cudaSuccess) e = launch_geometry(geo, georow, kap, binom, g.p.tau_lim, mmax, g.stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(g.stream);  // binom is still read
   dev_free(binom);
   if (e != cudaSuccess) {
@@ -296,8 +296,11 @@ struct RatesPlan {
 // / two / a face; 128^3): R = 12 (half-width 8), 4e4 sources 16.7 / 10.4 / 7.3 / 5.2;
 // R = 22 (15), 1e4: 7.4 / 4.7 / 4.0 / 3.7; R = 27 (19), 8e3: 7.7 / 5.1 / 4.7 / 5.8;
 // R = 33 (23), 5e3: 6.5 / 4.8 / 4.6 / -; R = 50 (35), 2e3: 5.8 / 5.3 / 7.0 / -; R = 60
-// (42), 1e3: 4.8 / 5.3 / - / -: hence the half-widths.  One quadrant
-// per warp is launched twice, as its warps' shared memory goes by the widest source: from
+// (42), 1e3: 4.8 / 5.3 / - / -: hence the half-widths, but for two quadrants: since one
+// runs 21 warps per SM it takes at R = 33 what two take (4.22 / 4.28), in an ionised box
+// (1.5e3 sources) 4.88 / 5.62, with the early exit 0.41 / 0.45; at R = 27 5.17 / 5.03, 5.51 /
+// 5.57 and 0.75 / 0.71.  With optical-depth weights two never pay (2e3 sources of R =
+// 5..50: 2.77 ms with them, 2.54 without).  One quadrant per warp is launched twice, as its warps' shared memory goes by the widest source: from
 // half-width 30 on 14 warps fit an SM, below 21 (250^3, 3e5 sources of R = 5..50: 143.4 /
 // 138.2 ms in four launches; 128^3, 1.6e4 7.26 / 7.21, with the early exit 1.18 / 1.28;
 // 64^3, 1e3 0.47 / 0.54: only where both parts are large).  A launch pays for its last
@@ -335,7 +338,10 @@ static RatesPlan rates_plan(const Grid& g, const int* r2s, int ns, bool exit) {
     for (int k = 1; k < K; ++k) p.cut[k] = ns;
     return p;
   }
-  const int lim[K] = {0, exit && longest_part(g, 24) > 0.1 ? 19 : 38, 30, 23, g.ftab ? 16 : 0};
+  const int face = g.ftab ? 16 : 0;
+  const bool od = g.interp_mode == RT_INTERP_OPTICAL_DEPTH;
+  if (od) p.mode[3] = 1;
+  const int lim[K] = {0, exit && longest_part(g, 24) > 0.1 ? 19 : 38, 30, od ? face : 20, face};
   for (int k = 1; k < K; ++k) p.cut[k] = std::max(p.cut[k - 1], first_fitting(g, r2s, ns, lim[k]));
   for (int k = K - 1; k > 1; --k) {
     double items = 24.0 / p.mode[k] * (p.cut[k + 1] - p.cut[k]);

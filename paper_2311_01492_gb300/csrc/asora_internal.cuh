@@ -46,11 +46,11 @@ inline int64_t geo_count(int mmax) { return geo_index(mmax + 1, 0, 0); }
 // Row-major geometry for the batched trace: entry (m, a1, a2), 0 <= a1, a2 <= m,
 // holds the weights in the cell's own orientation (a = a1/m, b = a2/m):
 //   w1 = (1-a)(1-b), w2 = a(1-b), w3 = (1-a)b, w4 = ab, ds = sqrt(1 + (a1^2+a2^2)/m^2),
-//   invv, thin as in GeoEntry
+//   invv, thin as in GeoEntry, lim: the largest dtau with dtau ds <= tau_lim
 // (bit-identical to the (lo, hi) table's values; consecutive a2 are adjacent).
 struct __align__(16) GeoRow {
   double w1, w2, w3, w4;
-  double ds, pad, invv, thin;
+  double ds, lim, invv, thin;
 };
 __host__ __device__ inline int64_t georow_index(int m, int a1, int a2) {
   return (int64_t)m * (m + 1) * (2 * m + 1) / 6 - 1 + (int64_t)a1 * (m + 1) + a2;
@@ -315,7 +315,8 @@ cudaError_t launch_tau_to_coldens(Grid& g, double* coldens);
 // gamma += thick / n_HI where thick != 0
 cudaError_t launch_add_thick(Grid& g, double* gamma, const int* skip);
 cudaError_t launch_validate_fields(Grid& g, const double* nH, const double* xHI);
-cudaError_t launch_geometry(GeoEntry* geo, GeoRow* georow, double* kap, double2* binom, int mmax,
+cudaError_t launch_geometry(GeoEntry* geo, GeoRow* georow, double* kap, double2* binom,
+                            double tau_lim, int mmax,
                             cudaStream_t s);
 cudaError_t launch_trace_faces(Grid& g, const TraceArgs& a, int block, int grid, size_t smem,
                                int wpb = 8);  // wpb: warps per CTA in warp mode (block 32)

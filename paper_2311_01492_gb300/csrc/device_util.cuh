@@ -24,6 +24,16 @@ __device__ __forceinline__ uint64_t bits_of(double x) {
   return (uint64_t)__double_as_longlong(x);
 }
 
+// x != 0 and max(x, y) for x, y >= +0 (NaN x: y) without an FP64 instruction: comparing
+// doubles takes as long as multiplying them.
+__device__ __forceinline__ bool nonzero(double x) {
+  return ((__double2hiint(x) << 1) | __double2loint(x)) != 0;
+}
+__device__ __forceinline__ double max_pos(double x, double y) {
+  const uint64_t b = bits_of(x);
+  return b > bits_of(y) && b <= 0x7ff0000000000000ull ? x : y;
+}
+
 // Chord table lookup: segment from the IEEE bits of tau (tau >= +0).
 __device__ __forceinline__ double tab_eval(const double2* __restrict__ t, const TabDev& tb,
                                            double tau) {
@@ -38,6 +48,25 @@ __device__ __forceinline__ double tab_eval(const double2* __restrict__ t, const 
   }
   const double2 c = __ldg(&t[seg]);
   return fma(c.y, tau, c.x);
+}
+
+// The chord c0 + c1 tau of tau's segment (not for exact grey opacity); zeros beyond the
+// table.
+struct Chord {
+  double c0, c1, tau;
+};
+__device__ __forceinline__ Chord tab_chord(const double2* __restrict__ t, const TabDev& tb,
+                                           double tau) {
+  const uint64_t b = bits_of(tau);
+  if (b >= tb.tau_max_bits) return {0.0, 0.0, 0.0};
+  int seg = 0;
+  if (b >= tb.tau_min_bits) {
+    const int e = (int)(b >> 52) - 1023;
+    const int m = (int)((b >> (52 - tb.B)) & (uint64_t)((1 << tb.B) - 1));
+    seg = 1 + ((e + tb.E0) << tb.B) + m;
+  }
+  const double2 c = __ldg(&t[seg]);
+  return {c.x, c.y, tau};
 }
 
 // Rate of one cell (photon-conserving, Eq. sugg; thin limit Eq. gammalocal).
@@ -68,7 +97,7 @@ __device__ __forceinline__ double od_interp_r(double w1, double w2, double w3, d
   return quick_div(fma(v4, c4, fma(v3, c3, fma(v2, c2, fma(v1, c1, nz)))), S);
 }
 __device__ __forceinline__ double od_recip(double c, double tw0) {
-  return quick_recip(fmax(c, tw0));
+  return quick_recip(max_pos(c, tw0));
 }
 __device__ __forceinline__ double od_interp(double w1, double w2, double w3, double w4, double c1,
                                             double c2, double c3, double c4, double tw0,

@@ -206,7 +206,8 @@ __global__ void k_geometry(GeoEntry* __restrict__ geo, int mmax) {
 // Row-major entry (m, a1, a2) with the same correctly rounded expressions.
 __global__ void k_geometry_rows(GeoRow* __restrict__ geo, double* __restrict__ kap,
                                 double* __restrict__ kappa, double* __restrict__ ikappa,
-                                double* __restrict__ dsik, const double2* __restrict__ binom, int mmax) {
+                                double* __restrict__ dsik, const double2* __restrict__ binom, double tau_lim,
+                                int mmax) {
   const int m = blockIdx.x + 1;
   if (m > mmax) return;
   const int cnt = (m + 1) * (m + 1);
@@ -220,7 +221,13 @@ __global__ void k_geometry_rows(GeoRow* __restrict__ geo, double* __restrict__ k
     e.w3 = (1.0 - x) * y;
     e.w4 = x * y;
     e.ds = sqrt(1.0 + (double)(a1 * a1 + a2 * a2) / (double)(m * m));
-    e.pad = 0.0;
+    e.lim = tau_lim / e.ds;  // the bound itself is a step or two away at most
+    for (int k = 0; k < 4 && e.lim * e.ds > tau_lim; ++k)
+      e.lim = __longlong_as_double(__double_as_longlong(e.lim) - 1);
+    for (int k = 0; k < 4; ++k) {
+      const double up = __longlong_as_double(__double_as_longlong(e.lim) + 1);
+      if (up * e.ds <= tau_lim) e.lim = up;
+    }
     const double r2 = (double)(m * m + a1 * a1 + a2 * a2);
     const double fourpi = 12.566370614359172;
     e.invv = 1.0 / (fourpi * r2 * e.ds);
@@ -240,13 +247,14 @@ __global__ void k_geometry_rows(GeoRow* __restrict__ geo, double* __restrict__ k
 
 // k = min(mmax, kKapMax): binom is scratch of (k + 1)(k + 2)/2 double2, kap holds
 // georow_count(k) values of kappa ds, then as many of kappa, 1/kappa and ds/kappa
-cudaError_t launch_geometry(GeoEntry* geo, GeoRow* georow, double* kap, double2* binom, int mmax,
-                            cudaStream_t s) {
+cudaError_t launch_geometry(GeoEntry* geo, GeoRow* georow, double* kap, double2* binom,
+                            double tau_lim, int mmax, cudaStream_t s) {
   if (mmax < 1) return cudaSuccess;
   k_binomials<<<std::min(mmax, kKapMax) + 1, 64, 0, s>>>(binom, std::min(mmax, kKapMax));
   count_launch();
   const int64_t nk = georow_count(std::min(mmax, kKapMax));
-  k_geometry_rows<<<mmax, 256, 0, s>>>(georow, kap, kap + nk, kap + 2 * nk, kap + 3 * nk, binom, mmax);
+  k_geometry_rows<<<mmax, 256, 0, s>>>(georow, kap, kap + nk, kap + 2 * nk, kap + 3 * nk, binom,
+                                         tau_lim, mmax);
   count_launch();
   k_geometry<<<mmax, 256, 0, s>>>(geo, mmax);
   count_launch();

@@ -107,7 +107,7 @@ __device__ __forceinline__ void trace_face_item(const TraceArgs& a, const int it
         dG = nd * ((tab_eval(a.tab.g, a.tab, 0.0) - tab_eval(a.tab.g, a.tab, tout)) *
                    B.inv_cell3 * a.invn[scell]);
       ++nrate;
-      if (dG != 0.0) atomicAdd(&a.gamma[scell], dG);
+      if (nonzero(dG)) atomicAdd(&a.gamma[scell], dG);
     }
   }
 
@@ -199,7 +199,7 @@ __device__ __forceinline__ void trace_face_item(const TraceArgs& a, const int it
         const double dG = cell_rate(a, nd * B.inv_cell3, nd * B.thin_fac, tin, tout, dcell, ge,
                                     &a.invn[cell]);
         ++nrate;
-        if (dG != 0.0) atomicAdd(&a.gamma[cell], dG);
+        if (nonzero(dG)) atomicAdd(&a.gamma[cell], dG);
       }
     }
   };
@@ -341,7 +341,7 @@ __device__ __forceinline__ void trace_face_item(const TraceArgs& a, const int it
             const double dG = cell_rate(a, nd * B.inv_cell3, nd * B.thin_fac, tin, tout, dcell, ge,
                                         &a.invn[cell]);
             ++nrate;
-            if (dG != 0.0) atomicAdd(&a.gamma[cell], dG);
+            if (nonzero(dG)) atomicAdd(&a.gamma[cell], dG);
           }
         }
       }
@@ -490,7 +490,7 @@ __device__ __forceinline__ void trace_face_whole(const TraceArgs& a, const int i
         dG = nd * ((tab_eval(a.tab.g, a.tab, 0.0) - tab_eval(a.tab.g, a.tab, tout)) *
                    B.inv_cell3 * a.invn[scell]);
       ++nrate;
-      if (dG != 0.0) atomicAdd(&a.gamma[scell], dG);
+      if (nonzero(dG)) atomicAdd(&a.gamma[scell], dG);
     }
   }
 
@@ -607,7 +607,7 @@ __device__ __forceinline__ void trace_face_whole(const TraceArgs& a, const int i
             const double dG = cell_rate(a, nd * B.inv_cell3, nd * B.thin_fac, tin, tout, dcell, ge,
                                         &a.invn[cell]);
             ++nrate;
-            if (dG != 0.0) atomicAdd(&a.gamma[cell], dG);
+            if (nonzero(dG)) atomicAdd(&a.gamma[cell], dG);
           }
         }
       }
@@ -858,7 +858,7 @@ __global__ void __launch_bounds__(BLOCK) k_trace_shells(TraceArgs a) {
               else
                 dG = nd * ((tab_eval(a.tab.g, a.tab, 0.0) - tab_eval(a.tab.g, a.tab, tout)) *
                            B.inv_cell3 * a.invn[cell]);
-              if (dG != 0.0) atomicAdd(&a.gamma[cell], dG);
+              if (nonzero(dG)) atomicAdd(&a.gamma[cell], dG);
             }
             continue;
           }
@@ -906,7 +906,7 @@ __global__ void __launch_bounds__(BLOCK) k_trace_shells(TraceArgs a) {
             const double dG = cell_rate(a, nd * B.inv_cell3, nd * B.thin_fac, tin, tout, dcell, ge,
                                         &a.invn[cell]);
             ++nrate;
-            if (dG != 0.0) atomicAdd(&a.gamma[cell], dG);
+            if (nonzero(dG)) atomicAdd(&a.gamma[cell], dG);
           }
         }
       };
