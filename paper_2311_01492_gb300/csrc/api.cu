@@ -85,12 +85,12 @@ static int isqrt_h(int64_t x) {
 }
 
 static void free_grid(Grid* g) {
-  dev_free(g->boxes_d); dev_free(g->gtab); dev_free(g->htab);
+  dev_free(g->small); cudaFreeHost(g->pin); dev_free(g->gtab); dev_free(g->htab);
   dev_free(g->dtau); dev_free(g->dtauT); dev_free(g->invn);
   free_sources(*g);
-  dev_free(g->geo); dev_free(g->georow); dev_free(g->kap); dev_free(g->queue); dev_free(g->err);
-  dev_free(g->cube); dev_free(g->od_scratch); dev_free(g->unconv); dev_free(g->xbuf); dev_free(g->xavg);
-  dev_free(g->xavg2); dev_free(g->xhi_int); dev_free(g->flags); dev_free(g->counters);
+  dev_free(g->geo); dev_free(g->georow); dev_free(g->kap);
+  dev_free(g->cube); dev_free(g->od_scratch); dev_free(g->xbuf); dev_free(g->xavg);
+  dev_free(g->xavg2); dev_free(g->xhi_int);
   dev_free(g->bwd_stack); dev_free(g->dq_merged); dev_free(g->bwd_redo);
   free_row_tables(*g);
   if (g->it_exec) cudaGraphExecDestroy(g->it_exec);
@@ -121,13 +121,10 @@ static rt_status ensure_geometry(Grid& g, int mmax) {
   TRY(dev_malloc(&geo, geo_count(mmax) * sizeof(GeoEntry)));
   const int kmax = std::min(mmax, kKapMax);
   double* kap = nullptr;
-  double2* binom = nullptr;
+  const size_t nkap = 4 * georow_count(kmax) + (size_t)(kmax + 1) * (kmax + 2);
   cudaError_t e = dev_malloc(&georow, georow_count(mmax) * sizeof(GeoRow));
-  if (e == cudaSuccess) e = dev_malloc(&kap, 4 * georow_count(kmax) * sizeof(double));
-  if (e == cudaSuccess) e = dev_malloc(&binom, (size_t)(kmax + 1) * (kmax + 2) / 2 * sizeof(double2));
-  if (e == cudaSuccess) e = launch_geometry(geo, georow, kap, binom, g.p.tau_lim, mmax, g.stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(g.stream);  // binom is still read
-  dev_free(binom);
+  if (e == cudaSuccess) e = dev_malloc(&kap, nkap * sizeof(double));
+  if (e == cudaSuccess) e = launch_geometry(geo, georow, kap, g.p.tau_lim, mmax, g.stream);
   if (e != cudaSuccess) {
     dev_free(geo);
     dev_free(georow);
@@ -213,13 +210,15 @@ static TraceArgs base_args(Grid& g) {
   return a;
 }
 
-// Error bits latched by the kernels since the last check (the caller has
-// synchronised the grid's stream); clears them.
+// Synchronises the grid's stream; error bits latched by the kernels since the last check,
+// cleared.
 static rt_status latched_errors(Grid& g) {
-  int herr = 0;
-  TRY(cudaMemcpy(&herr, g.err, sizeof(int), cudaMemcpyDeviceToHost));
+  TRY(cudaMemcpyAsync(g.pin + 1, g.err, sizeof(int), cudaMemcpyDeviceToHost, g.stream));
+  TRY(cudaStreamSynchronize(g.stream));
+  const int herr = g.pin[1];
   if (!herr) return RT_OK;
-  TRY(cudaMemset(g.err, 0, sizeof(int)));
+  TRY(cudaMemsetAsync(g.err, 0, sizeof(int), g.stream));
+  TRY(cudaStreamSynchronize(g.stream));
   std::string what;
   if (herr & ERR_LAYER_CAP) what += " layer wider than the shared-memory capacity;";
   if (herr & ERR_GEO) what += " layer beyond the geometry table;";
@@ -362,7 +361,7 @@ struct RatesLaunch {
   int mode, hcap, begin, end, grid, wpb;  // items [begin, end)
   size_t smem;
 };
-static rt_status rates_launches(const Grid& g, bool exit, std::vector<RatesLaunch>& out) {
+static rt_status rates_launches(Grid& g, bool exit, std::vector<RatesLaunch>& out) {
   const int* r2s = g.r2_sorted_h.data();
   const RatesPlan plan = rates_plan(g, r2s, g.nsrc, exit);
   const bool od = g.interp_mode == RT_INTERP_OPTICAL_DEPTH;
@@ -379,21 +378,29 @@ static rt_status rates_launches(const Grid& g, bool exit, std::vector<RatesLaunc
       return fail(RT_ERR_INVALID, "rt_raytrace: radius too large for the batched schedule's "
                                   "shared-memory layers; use RT_SCHED_PLAIN");
     L.wpb = 1;
-    int maxg = 0;
-    if (k == 0) {
-      maxg = rates_max_grid(L.mode, L.smem, 1, exit, od);
-    } else {
-      // CTAs of as many warps as keeps the most resident (a warp's shared memory grows
-      // with its layer capacity, and every CTA also reserves some; ties go to the
-      // larger CTA)
-      for (int cand = rates_max_warps(L.mode, exit, od); cand >= 1; --cand) {
-        const int mg = rates_max_grid(L.mode, L.smem * cand, cand, exit, od);
-        if (mg * cand > maxg * L.wpb) {
-          maxg = mg;
-          L.wpb = cand;
+    // (kept per grid: what fits an SM does not change, and asking takes 10 us a trace)
+    const std::array<int, 4> key{L.mode, L.hcap, exit, od};
+    auto fits = g.occupancy.find(key);
+    if (fits == g.occupancy.end()) {
+      int maxg = 0;
+      if (k == 0) {
+        maxg = rates_max_grid(L.mode, L.smem, 1, exit, od);
+      } else {
+        // CTAs of as many warps as keeps the most resident (a warp's shared memory grows
+        // with its layer capacity, and every CTA also reserves some; ties go to the
+        // larger CTA)
+        for (int cand = rates_max_warps(L.mode, exit, od); cand >= 1; --cand) {
+          const int mg = rates_max_grid(L.mode, L.smem * cand, cand, exit, od);
+          if (mg * cand > maxg * L.wpb) {
+            maxg = mg;
+            L.wpb = cand;
+          }
         }
       }
+      if (maxg > 0) fits = g.occupancy.emplace(key, std::make_pair(maxg, L.wpb)).first;
     }
+    const int maxg = fits == g.occupancy.end() ? 0 : fits->second.first;
+    if (maxg > 0) L.wpb = fits->second.second;
     if (maxg <= 0) return fail(RT_ERR_CUDA, "rt_raytrace: no occupancy for a rate kernel");
     const int n = L.end - L.begin;
     L.grid = L.mode & kAhead ? n : std::max(1, std::min((n + L.wpb - 1) / L.wpb, maxg));
@@ -407,7 +414,6 @@ static rt_status run_rates(Grid& g, const TraceArgs& a, const int* items) {
   std::vector<RatesLaunch> ls;
   rt_status st = rates_launches(g, a.early_exit != 0, ls);
   if (st != RT_OK) return st;
-  TRY(cudaMemsetAsync(g.queue, 0, RatesPlan::kClasses * sizeof(int), g.stream));
   for (size_t k = 0; k < ls.size(); ++k) {
     const RatesLaunch& L = ls[k];
     TraceArgs b = a;
@@ -439,7 +445,7 @@ static rt_status run_trace(Grid& g, double* gamma, double* coldens, const int* i
   a.skip = skip;
   a.early_exit = early_exit ? 1 : 0;
   g.stats.launches = 0;
-  TRY(cudaMemsetAsync(g.counters, 0, sizeof(unsigned long long), g.stream));
+  TRY(cudaMemsetAsync(g.counters, 0, 64 + 8 * sizeof(int), g.stream));  // and the queues
   const bool od = a.interp_mode == RT_INTERP_OPTICAL_DEPTH;
   const bool rates = gamma && takes_rates_kernels(g, early_exit);
   if (schedule != RT_SCHED_PLAIN && g.nmax > 1290)
@@ -454,7 +460,6 @@ static rt_status run_trace(Grid& g, double* gamma, double* coldens, const int* i
     a.hcap = E;
     a.items = items;
     a.n_items = nsrc_plain;
-    TRY(cudaMemsetAsync(g.queue, 0, sizeof(int), g.stream));
     TRY(launch_trace_shells(g, a, block, grid));
     g.stats.block = block;
     g.stats.grid = grid;
@@ -476,7 +481,6 @@ static rt_status run_trace(Grid& g, double* gamma, double* coldens, const int* i
     const int pw = first_fitting(g, r2s, ns, g.hsmall);
     const int p4 = std::max(pw, first_fitting(g, r2s, ns, g.hface));
     const int hbig = face_hcap(r2s[0], g.nmax);
-    TRY(cudaMemsetAsync(g.queue, 0, 3 * sizeof(int), g.stream));
     a.items = items;
     g.stats.launches = 0;
     // warp modes: CTAs of 1..8 warps, whichever keeps the most warps resident (a
@@ -595,18 +599,25 @@ rt_status rt_ensemble_create(rt_grid_t* out, int nbox, const int* h_n, const dou
   }
   g->ncell = off;
   cudaError_t e = cudaSuccess;
-  e = dev_malloc(&g->boxes_d, nbox * sizeof(BoxDev));
-  if (e == cudaSuccess) e = cudaMemcpy(g->boxes_d, g->boxes_h.data(), nbox * sizeof(BoxDev), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = dev_malloc(&g->dtau, g->ncell * sizeof(double));
+  e = dev_malloc(&g->dtau, g->ncell * sizeof(double));
   if (e == cudaSuccess) e = dev_malloc(&g->dtauT, g->ncell * sizeof(double));
   if (e == cudaSuccess) e = dev_malloc(&g->invn, g->ncell * sizeof(double));
-  if (e == cudaSuccess) e = dev_malloc(&g->queue, 64 * sizeof(int));
-  if (e == cudaSuccess) e = dev_malloc(&g->err, 2 * sizeof(int));  // [0] traces, [1] validation
-  if (e == cudaSuccess) e = cudaMemset(g->err, 0, 2 * sizeof(int));
-  if (e == cudaSuccess) e = dev_malloc(&g->unconv, 16 * sizeof(int64_t));
-  if (e == cudaSuccess) e = dev_malloc(&g->flags, 16 * sizeof(int));
-  if (e == cudaSuccess) e = dev_malloc(&g->counters, 8 * sizeof(unsigned long long));
-  if (e == cudaSuccess) e = cudaMemset(g->counters, 0, 8 * sizeof(unsigned long long));
+  // the small arrays: counters 0 (8), queue 64 (64 ints: the counters and the first 8 are
+  // cleared together), err 320, flags 384 (16 ints), unconv 448 (16 64-bit counts), boxes 576
+  const size_t small = 576 + nbox * sizeof(BoxDev);
+  if (e == cudaSuccess) e = dev_malloc(&g->small, small);
+  if (e == cudaSuccess) {
+    g->counters = reinterpret_cast<unsigned long long*>(g->small);
+    g->queue = reinterpret_cast<int*>(g->small + 64);
+    g->err = reinterpret_cast<int*>(g->small + 320);
+    g->flags = reinterpret_cast<int*>(g->small + 384);
+    g->unconv = reinterpret_cast<int64_t*>(g->small + 448);
+    g->boxes_d = reinterpret_cast<BoxDev*>(g->small + 576);
+    std::vector<char> up(small, 0);
+    memcpy(up.data() + 576, g->boxes_h.data(), nbox * sizeof(BoxDev));
+    e = cudaMemcpy(g->small, up.data(), small, cudaMemcpyHostToDevice);
+  }
+  if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&g->pin), kPinBytes);
   for (auto& ev : g->ev)
     if (e == cudaSuccess) e = cudaEventCreate(&ev);
   if (e != cudaSuccess) {
@@ -688,12 +699,10 @@ static rt_status set_field(rt_grid_t h, const double* d, bool density) {
   if (!h) return fail(RT_ERR_INVALID, std::string(who) + ": null grid");
   if (!d) return fail(RT_ERR_INVALID, std::string(who) + ": null field");
   Grid& g = *reinterpret_cast<Grid*>(h);
-  int herr = 0;
-  TRY(cudaMemsetAsync(g.err + 1, 0, sizeof(int), g.stream));
+  g.pin[0] = 0;
   TRY(launch_validate_fields(g, density ? d : nullptr, density ? nullptr : d));
-  TRY(cudaMemcpyAsync(&herr, g.err + 1, sizeof(int), cudaMemcpyDeviceToHost, g.stream));
   TRY(cudaStreamSynchronize(g.stream));
-  if (herr)
+  if (g.pin[0])
     return fail(RT_ERR_INVALID, density ? "rt_set_density: n_H must be finite, >= +0 and <= 1e12"
                                         : "rt_set_xHI: x_HI must lie in [+0, 1]");
   if (density) g.nH = d; else g.xHI = d;
@@ -800,7 +809,6 @@ rt_status rt_raytrace_source_coldens(rt_grid_t h, int src, double* d_coldens, in
     g.stats.grid = 24;
     g.stats.items = 24;
     g.stats.schedule = RT_SCHED_BATCHED;
-    TRY(cudaStreamSynchronize(g.stream));
     return latched_errors(g);
   }
   int p = 0;
@@ -842,7 +850,6 @@ rt_status rt_get_stats(rt_grid_t h, rt_stats* out) {
 rt_status rt_check(rt_grid_t h) {
   if (!h) return fail(RT_ERR_INVALID, "rt_check: null grid");
   Grid& g = *reinterpret_cast<Grid*>(h);
-  TRY(cudaStreamSynchronize(g.stream));
   return latched_errors(g);
 }
 
@@ -986,12 +993,10 @@ rt_status rt_iterate(rt_grid_t h, double* d_x, double dt_s, double alpha_H, doub
   }
   TRY(cudaMemcpyAsync(d_x, g.xbuf, bytes, cudaMemcpyDeviceToDevice, user));
   if (h_iters) {
-    int fl[2] = {0, 0};
-    TRY(cudaMemcpyAsync(fl, g.flags, 2 * sizeof(int), cudaMemcpyDeviceToHost, user));
-    TRY(cudaStreamSynchronize(user));
-    iters = fl[1];
-    *h_iters = iters;
-    return latched_errors(g);
+    TRY(cudaMemcpyAsync(g.pin + 2, g.flags, 2 * sizeof(int), cudaMemcpyDeviceToHost, user));
+    const rt_status err = latched_errors(g);  // (synchronises)
+    *h_iters = iters = g.pin[3];
+    return err;
   }
   return RT_OK;
 }

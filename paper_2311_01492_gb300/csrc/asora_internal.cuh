@@ -4,8 +4,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <string>
+#include <array>
 #include <map>
+#include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/asora.h"
@@ -56,6 +58,8 @@ __host__ __device__ inline int64_t georow_index(int m, int a1, int a2) {
   return (int64_t)m * (m + 1) * (2 * m + 1) / 6 - 1 + (int64_t)a1 * (m + 1) + a2;
 }
 inline int64_t georow_count(int mmax) { return georow_index(mmax + 1, 0, 0); }
+
+constexpr size_t kPinBytes = 1 << 16;  // of Grid::pin
 
 // kappa = C(m, a1) C(m, a2) and kappa ds for the batched rates (rates.cu), at
 // georow_index(m, a1, a2), for layers m <= kKapMax (no layer that the batched
@@ -191,16 +195,18 @@ struct Grid {
     int* mr2 = nullptr;
     uint32_t *lkey = nullptr, *lkey2 = nullptr;
     int *lval = nullptr, *order = nullptr, *lpt = nullptr;
-    void* tmp = nullptr;
+    char* tmp = nullptr;
+    char* arena = nullptr;     // holds all of the above, and the ingested sources
+    void* pinned = nullptr;    // holds the host arrays below
     size_t tmp_bytes = 0;
     int* dscal = nullptr;      // device scalars: [0] largest r2
-    int* hscal = nullptr;      // pinned host: error bits, last head, last offset, largest r2
     int* r2pin = nullptr;      // pinned host: r2 per merged source
     SrcDev* srcpin = nullptr;  // pinned host: merged sources (ensembles)
   } ing;
 
   // precomputed row tables of the batched trace (see TraceArgs::rtab)
   unsigned char* rtab = nullptr;
+  char* tables = nullptr;  // holds the row, interior and face tables and what describes them
   int* rtab_off = nullptr;
   int* rtab_first = nullptr;
   int* rtab_hcap = nullptr;
@@ -226,8 +232,13 @@ struct Grid {
   int kap_mmax = 0;
 
   // scratch
+  char* small = nullptr;  // holds boxes_d, counters, queue, err, flags, unconv
   int* queue = nullptr;
   int* err = nullptr;
+  int* pin = nullptr;  // pinned host words that kernels and copies write: [0] validation of
+                       // inputs, [1] err, [2, 3] flags, [4, 5] merged sources and largest r2;
+                       // from byte 64 of kPinBytes: the ingest's arrays, if they fit
+  std::map<std::array<int, 4>, std::pair<int, int>> occupancy;  // of the rate kernels
   double* cube = nullptr;       // shell-kernel scratch
   double* od_scratch = nullptr; // reciprocals of the batched rates with mode 1
   size_t cube_bytes = 0;
@@ -315,8 +326,7 @@ cudaError_t launch_tau_to_coldens(Grid& g, double* coldens);
 // gamma += thick / n_HI where thick != 0
 cudaError_t launch_add_thick(Grid& g, double* gamma, const int* skip);
 cudaError_t launch_validate_fields(Grid& g, const double* nH, const double* xHI);
-cudaError_t launch_geometry(GeoEntry* geo, GeoRow* georow, double* kap, double2* binom,
-                            double tau_lim, int mmax,
+cudaError_t launch_geometry(GeoEntry* geo, GeoRow* georow, double* kap, double tau_lim, int mmax,
                             cudaStream_t s);
 cudaError_t launch_trace_faces(Grid& g, const TraceArgs& a, int block, int grid, size_t smem,
                                int wpb = 8);  // wpb: warps per CTA in warp mode (block 32)

@@ -6,7 +6,9 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <map>
+#include <type_traits>
 
 #include "asora_internal.cuh"
 #include "device_util.cuh"
@@ -14,8 +16,7 @@
 namespace asora {
 
 // ----------------------------------------------------------- validation
-// (writes its own error word, g.err[1], so that it never clears the bits the
-// trace kernels latch in g.err[0])
+// (writes its own error word, so that it never clears the bits the trace kernels latch)
 __global__ void k_validate_fields(const BoxDev* __restrict__ boxes, int nbox,
                                   const double* __restrict__ nH, const double* __restrict__ xHI,
                                   int64_t ncell, int* __restrict__ err) {
@@ -31,11 +32,11 @@ __global__ void k_validate_fields(const BoxDev* __restrict__ boxes, int nbox,
       if (!(v >= 0.0) || !(v <= 1.0) || signbit(v)) bad = 1;
     }
   }
-  if (bad) atomicOr(err, ERR_INPUT);
+  if (bad) *err = ERR_INPUT;  // (pinned host memory: nothing to clear or to copy back)
 }
 
 cudaError_t launch_validate_fields(Grid& g, const double* nH, const double* xHI) {
-  k_validate_fields<<<1024, 256, 0, g.stream>>>(g.boxes_d, g.nbox, nH, xHI, g.ncell, g.err + 1);
+  k_validate_fields<<<1024, 256, 0, g.stream>>>(g.boxes_d, g.nbox, nH, xHI, g.ncell, g.pin);
   count_launch();
   return cudaGetLastError();
 }
@@ -245,11 +246,12 @@ __global__ void k_geometry_rows(GeoRow* __restrict__ geo, double* __restrict__ k
   }
 }
 
-// k = min(mmax, kKapMax): binom is scratch of (k + 1)(k + 2)/2 double2, kap holds
-// georow_count(k) values of kappa ds, then as many of kappa, 1/kappa and ds/kappa
-cudaError_t launch_geometry(GeoEntry* geo, GeoRow* georow, double* kap, double2* binom,
-                            double tau_lim, int mmax, cudaStream_t s) {
+// k = min(mmax, kKapMax): kap holds georow_count(k) values of kappa ds, then as many of
+// kappa, 1/kappa and ds/kappa, then scratch: the binomials
+cudaError_t launch_geometry(GeoEntry* geo, GeoRow* georow, double* kap, double tau_lim, int mmax,
+                            cudaStream_t s) {
   if (mmax < 1) return cudaSuccess;
+  double2* binom = reinterpret_cast<double2*>(kap + 4 * georow_count(std::min(mmax, kKapMax)));
   k_binomials<<<std::min(mmax, kKapMax) + 1, 64, 0, s>>>(binom, std::min(mmax, kKapMax));
   count_launch();
   const int64_t nk = georow_count(std::min(mmax, kKapMax));
@@ -281,11 +283,18 @@ __global__ void k_src_keys(const BoxDev* __restrict__ boxes, int nbox, int nsrc,
   const double cap = 3.0 * (double)(B.n / 2) * (double)(B.n / 2) + 1.0;
   const double rr = fmin(floor(R * R), cap);
   const int r2 = bad ? 0 : (int)rr;
-  if (bad) atomicOr(err, ERR_INPUT);
+  if (bad) *err = ERR_INPUT;
   const int64_t cell = bad ? 0 : B.off + ((int64_t)i * B.n + j) * B.n + k;
   keys[s] = ((uint64_t)cell << 22) | (uint64_t)r2;
   idx[s] = s;
   r2out[s] = r2;
+}
+
+// Number of merged sources and the largest r2, to pinned host memory.
+__global__ void k_src_scalars(const int* __restrict__ last_head, const int* __restrict__ last_mid,
+                              const int* __restrict__ max_r2, int* __restrict__ out) {
+  out[0] = *last_head + *last_mid;
+  out[1] = *max_r2;
 }
 
 __global__ void k_src_heads(const uint64_t* __restrict__ keys, int nsrc, int* __restrict__ head) {
@@ -373,47 +382,25 @@ static int64_t ball_count(int r2, int n) {
 
 void free_sources(Grid& g) {
   Grid::Ingest& w = g.ing;
-  dev_free(g.src); dev_free(g.ndot); dev_free(g.r2lim); dev_free(g.items);
-  dev_free(g.src_of_input); dev_free(g.ndot_in);
+  dev_free(w.arena);
+  cudaFreeHost(w.pinned);
   g.src = nullptr; g.ndot = nullptr; g.r2lim = nullptr; g.items = nullptr;
   g.src_of_input = nullptr; g.ndot_in = nullptr;
   g.src_cap = 0;
-  dev_free(w.keys); dev_free(w.keys2); dev_free(w.idx); dev_free(w.idx2); dev_free(w.r2in);
-  dev_free(w.head); dev_free(w.mid); dev_free(w.msrc); dev_free(w.mndot); dev_free(w.mr2);
-  dev_free(w.lkey); dev_free(w.lkey2); dev_free(w.lval); dev_free(w.order); dev_free(w.lpt);
-  dev_free(w.tmp); dev_free(w.dscal);
-  cudaFreeHost(w.hscal); cudaFreeHost(w.r2pin); cudaFreeHost(w.srcpin);
   w = Grid::Ingest{};
 }
 
-// Grow the per-source arrays (ingest scratch and the ingested sources) to n sources.
+// Grow the per-source arrays (ingest scratch and the ingested sources) to n sources: one
+// allocation on the device, and at most one of pinned memory.
 static cudaError_t reserve_sources(Grid& g, size_t n) {
   Grid::Ingest& w = g.ing;
   if (n <= w.cap && n <= g.src_cap) return cudaSuccess;
   cudaStreamSynchronize(g.stream);  // earlier work may still read the old arrays
   free_sources(g);
-  cudaError_t e = cudaSuccess;
-  auto dm = [&](auto*& p, size_t bytes) {
-    if (e == cudaSuccess) e = dev_malloc(reinterpret_cast<void**>(&p), bytes);
-  };
-  dm(w.keys, n * sizeof(uint64_t)); dm(w.keys2, n * sizeof(uint64_t));
-  dm(w.idx, n * sizeof(int)); dm(w.idx2, n * sizeof(int)); dm(w.r2in, n * sizeof(int));
-  dm(w.head, n * sizeof(int)); dm(w.mid, n * sizeof(int));
-  dm(w.msrc, n * sizeof(SrcDev)); dm(w.mndot, n * sizeof(double)); dm(w.mr2, n * sizeof(int));
-  dm(w.lkey, n * sizeof(uint32_t)); dm(w.lkey2, n * sizeof(uint32_t));
-  dm(w.lval, n * sizeof(int)); dm(w.order, n * sizeof(int)); dm(w.lpt, n * sizeof(int));
-  dm(w.dscal, 4 * sizeof(int));
-  dm(g.src, n * sizeof(SrcDev)); dm(g.ndot, n * sizeof(double)); dm(g.r2lim, n * sizeof(int));
-  dm(g.items, 24 * n * sizeof(int)); dm(g.src_of_input, n * sizeof(int));
-  dm(g.ndot_in, n * sizeof(double));
-  if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&w.hscal), 4 * sizeof(int));
-  if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&w.r2pin), n * sizeof(int));
-  if (e == cudaSuccess && g.nbox > 1)
-    e = cudaMallocHost(reinterpret_cast<void**>(&w.srcpin), n * sizeof(SrcDev));
-  // CUB scratch for the largest of its three uses at n items
+  // CUB scratch for the largest of its uses at n items
   size_t need = 0, tb = 0;
-  if (e == cudaSuccess) e = cub::DeviceRadixSort::SortPairs(nullptr, need, w.keys, w.keys2, w.idx,
-                                                            w.idx2, (int)n, 0, 64, g.stream);
+  cudaError_t e = cub::DeviceRadixSort::SortPairs(nullptr, need, w.keys, w.keys2, w.idx, w.idx2,
+                                                  (int)n, 0, 64, g.stream);
   tb = std::max(tb, need);
   if (e == cudaSuccess) e = cub::DeviceScan::ExclusiveSum(nullptr, need, w.head, w.mid, (int)n,
                                                           g.stream);
@@ -424,7 +411,42 @@ static cudaError_t reserve_sources(Grid& g, size_t n) {
   if (e == cudaSuccess) e = cub::DeviceReduce::Max(nullptr, need, w.r2in, w.dscal, (int)n,
                                                    g.stream);
   tb = std::max(tb, need);
-  dm(w.tmp, tb);
+  size_t bytes = 0;
+  char* base = nullptr;
+  auto part = [&](auto*& p, size_t count) {  // (a first pass adds up, a second one places)
+    if (base) p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(base + bytes);
+    bytes += (count * sizeof(*p) + 255) & ~(size_t)255;
+  };
+  auto parts = [&]() {
+    bytes = 0;
+    part(w.keys, n); part(w.keys2, n); part(w.idx, n); part(w.idx2, n); part(w.r2in, n);
+    part(w.head, n); part(w.mid, n); part(w.msrc, n); part(w.mndot, n); part(w.mr2, n);
+    part(w.lkey, n); part(w.lkey2, n); part(w.lval, n); part(w.order, n); part(w.lpt, n);
+    part(w.dscal, 4); part(g.src, n); part(g.ndot, n); part(g.r2lim, n); part(g.items, 24 * n);
+    part(g.src_of_input, n); part(g.ndot_in, n); part(w.tmp, tb);
+  };
+  auto pinned = [&]() {
+    bytes = 0;
+    part(w.r2pin, n);
+    if (g.nbox > 1) part(w.srcpin, n);
+  };
+  if (e == cudaSuccess) {
+    parts();
+    e = dev_malloc(&w.arena, bytes);
+    base = w.arena;
+    if (base) parts();
+  }
+  if (e == cudaSuccess) {
+    base = nullptr;
+    pinned();
+    if (bytes <= kPinBytes - 64) {  // behind the grid's own words
+      base = reinterpret_cast<char*>(g.pin) + 64;
+    } else {
+      e = cudaMallocHost(&w.pinned, bytes);
+      base = static_cast<char*>(w.pinned);
+    }
+    if (e == cudaSuccess) pinned();
+  }
   if (e != cudaSuccess) {
     free_sources(g);
     return e;
@@ -449,9 +471,9 @@ rt_status ingest_sources(Grid& g, int nsrc, const int32_t* d_pos, const int32_t*
   if (nsrc == 0) return RT_OK;
   CK(reserve_sources(g, (size_t)nsrc));
 
-  CK(cudaMemsetAsync(g.err + 1, 0, sizeof(int), s));  // the validation word, not the trace's
+  g.pin[0] = 0;
   k_src_keys<<<nb, T, 0, s>>>(g.boxes_d, g.nbox, nsrc, d_pos, d_box, d_ndot, d_radius, w.keys,
-                              w.idx, w.r2in, g.err + 1);
+                              w.idx, w.r2in, g.pin);
   count_launch();
   CK(cudaGetLastError());
   // stable sort by (cell, r2): co-located sources with equal radius become adjacent
@@ -465,18 +487,17 @@ rt_status ingest_sources(Grid& g, int nsrc, const int32_t* d_pos, const int32_t*
   CK(cub::DeviceScan::ExclusiveSum(w.tmp, need, w.head, w.mid, nsrc, s));
   need = w.tmp_bytes;
   CK(cub::DeviceReduce::Max(w.tmp, need, w.r2in, w.dscal, nsrc, s));  // for the LPT key
-  CK(cudaMemcpyAsync(w.hscal + 0, g.err + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(w.hscal + 1, w.head + nsrc - 1, sizeof(int), cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(w.hscal + 2, w.mid + nsrc - 1, sizeof(int), cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(w.hscal + 3, w.dscal, sizeof(int), cudaMemcpyDeviceToHost, s));
+  k_src_scalars<<<1, 1, 0, s>>>(w.head + nsrc - 1, w.mid + nsrc - 1, w.dscal, g.pin + 4);
+  count_launch();
+  CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
-  if (w.hscal[0]) {
+  if (g.pin[0]) {
     st = fail(RT_ERR_INVALID, "rt_set_sources: source outside its box, bad box id, radius <= 0 "
                               "or non-finite/negative photon rate");
     goto done;
   }
-  nm = w.hscal[2] + w.hscal[1];
-  g.max_r2 = w.hscal[3];
+  nm = g.pin[4];
+  g.max_r2 = g.pin[5];
   CK(cudaMemcpyAsync(g.ndot_in, d_ndot, nsrc * sizeof(double), cudaMemcpyDeviceToDevice, s));
   k_src_merge<<<nb, T, 0, s>>>(w.keys2, w.idx2, w.head, w.mid, nsrc, d_pos, d_box, d_ndot, w.r2in,
                                w.msrc, w.mndot, w.mr2, w.lkey, w.lval, g.src_of_input, g.max_r2);
@@ -657,9 +678,8 @@ __global__ void k_face_tables(const int4* __restrict__ job, unsigned char* __res
 }
 
 void free_row_tables(Grid& g) {
-  dev_free(g.rtab); dev_free(g.rtab_off); dev_free(g.rtab_first); dev_free(g.rtab_hcap);
-  dev_free(g.rtab_slot); dev_free(g.rtab_lay); dev_free(g.ftab); dev_free(g.ftab_lay);
-  dev_free(g.itab); dev_free(g.itab_off);
+  dev_free(g.tables);
+  g.tables = nullptr;
   g.rtab = nullptr; g.rtab_off = g.rtab_first = g.rtab_hcap = g.rtab_slot = nullptr;
   g.rtab_lay = nullptr;
   g.ftab = nullptr; g.ftab_lay = nullptr;
@@ -700,12 +720,14 @@ rt_status ensure_row_tables(Grid& g) {
     for (int m = 1; m <= L; ++m) {
       const int64_t rem = (int64_t)v - (int64_t)m * m;
       const int H = std::min(m, isqrt_host(rem));
-      int64_t total = 0;
-      for (int r = 0; r <= H; ++r) total += std::min(H, isqrt_host(rem - (int64_t)r * r)) + 1;
       const int LA = std::min(H, m - 1);
-      int64_t itotal = 0;
-      for (int a1 = 1; a1 <= LA; ++a1)
-        itotal += std::max(0, std::min(std::min(H, isqrt_host(rem - (int64_t)a1 * a1)), m - 1));
+      int64_t total = 0, itotal = 0;
+      int w = isqrt_host(rem);  // of rem - r^2: falls as r grows
+      for (int r = 0; r <= H; ++r) {
+        while ((int64_t)w * w > rem - (int64_t)r * r) --w;
+        total += std::min(H, w) + 1;
+        if (r >= 1 && r <= LA) itotal += std::max(0, std::min(std::min(H, w), m - 1));
+      }
       hc = std::max(hc, H);
       ent_r2.push_back(v);
       ent_m.push_back(m);
@@ -756,8 +778,29 @@ rt_status ensure_row_tables(Grid& g) {
   const int maxv = r2s.front();
   std::vector<int> slot(maxv + 1, -1);
   for (size_t i = 0; i < r2s.size(); ++i) slot[r2s[i]] = (int)i;
+  // one allocation: what the host knows (one upload), then the tables the kernels fill
   int *d_r2 = nullptr, *d_m = nullptr;
   int4* d_jobs = nullptr;
+  std::vector<char> up;
+  size_t bytes = 0;
+  auto part = [&](auto*& p, size_t n) {  // (a first pass adds up, a second one places)
+    if (g.tables) p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(g.tables + bytes);
+    bytes += (n * sizeof(*p) + 15) & ~(size_t)15;
+  };
+  auto host = [&](auto*& p, const auto& v) {
+    if (!g.tables) {
+      up.resize(bytes + ((v.size() * sizeof(v[0]) + 15) & ~(size_t)15));
+      memcpy(up.data() + bytes, v.data(), v.size() * sizeof(v[0]));
+    }
+    part(p, v.size());
+  };
+  auto parts = [&]() {
+    bytes = 0;
+    host(g.rtab_lay, lay); host(g.ftab_lay, flay); host(d_jobs, jobs);
+    host(g.rtab_off, off); host(g.itab_off, ioff); host(g.rtab_first, first);
+    host(g.rtab_hcap, hcap); host(g.rtab_slot, slot); host(d_r2, ent_r2); host(d_m, ent_m);
+    part(g.rtab, cur); part(g.itab, icur); part(g.ftab, fcur + 16);
+  };
   cudaStream_t s = g.stream;
 #undef CK
 #define CK(x)                                   \
@@ -768,31 +811,10 @@ rt_status ensure_row_tables(Grid& g) {
       goto fail;                                \
     }                                           \
   } while (0)
-  CK(dev_malloc(&g.rtab, std::max<int64_t>(cur, 16)));
-  CK(dev_malloc(&g.rtab_off, off.size() * sizeof(int)));
-  CK(dev_malloc(&g.rtab_first, first.size() * sizeof(int)));
-  CK(dev_malloc(&g.rtab_hcap, hcap.size() * sizeof(int)));
-  CK(dev_malloc(&g.rtab_slot, slot.size() * sizeof(int)));
-  CK(dev_malloc(&g.rtab_lay, std::max<size_t>(lay.size(), 1) * sizeof(int4)));
-  CK(cudaMemcpyAsync(g.rtab_lay, lay.data(), lay.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
-  CK(dev_malloc(&g.ftab, std::max<int64_t>(fcur, 16)));
-  CK(dev_malloc(&g.ftab_lay, std::max<size_t>(flay.size(), 1) * sizeof(int4)));
-  CK(cudaMemcpyAsync(g.ftab_lay, flay.data(), flay.size() * sizeof(int4), cudaMemcpyHostToDevice,
-                     s));
-  CK(dev_malloc(&g.itab, std::max<int64_t>(icur, 16)));
-  CK(dev_malloc(&g.itab_off, ioff.size() * sizeof(int)));
-  CK(cudaMemcpyAsync(g.itab_off, ioff.data(), ioff.size() * sizeof(int), cudaMemcpyHostToDevice, s));
-  CK(dev_malloc(&d_r2, std::max(nent, 1) * sizeof(int)));
-  CK(dev_malloc(&d_m, std::max(nent, 1) * sizeof(int)));
-  CK(dev_malloc(&d_jobs, std::max<size_t>(jobs.size(), 1) * sizeof(int4)));
-  CK(cudaMemcpyAsync(d_jobs, jobs.data(), jobs.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(g.rtab_off, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(g.rtab_first, first.data(), first.size() * sizeof(int),
-                     cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(g.rtab_hcap, hcap.data(), hcap.size() * sizeof(int), cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(g.rtab_slot, slot.data(), slot.size() * sizeof(int), cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(d_r2, ent_r2.data(), nent * sizeof(int), cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(d_m, ent_m.data(), nent * sizeof(int), cudaMemcpyHostToDevice, s));
+  parts();
+  CK(dev_malloc(&g.tables, bytes));
+  parts();
+  CK(cudaMemcpyAsync(g.tables, up.data(), up.size(), cudaMemcpyHostToDevice, s));
   if (nent > 0) {
     k_row_tables<<<nent, 64, 0, s>>>(d_r2, d_m, g.rtab_off, g.rtab, nent);
     count_launch();
@@ -805,9 +827,6 @@ rt_status ensure_row_tables(Grid& g) {
     CK(cudaGetLastError());
   }
   CK(cudaStreamSynchronize(s));  // host vectors go out of scope
-  dev_free(d_r2);
-  dev_free(d_m);
-  dev_free(d_jobs);
   g.rtab_max_r2 = maxv;
   g.rtab_bytes = cur;
   g.itab_bytes = icur;
@@ -818,9 +837,6 @@ rt_status ensure_row_tables(Grid& g) {
   return RT_OK;
 fail:
   cudaStreamSynchronize(s);
-  dev_free(d_r2);
-  dev_free(d_m);
-  dev_free(d_jobs);
   free_row_tables(g);
   return st;
 #undef CK
