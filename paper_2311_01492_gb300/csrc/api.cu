@@ -304,7 +304,9 @@ struct RatesPlan {
 // 138.2 ms in four launches; 128^3, 1.6e4 7.26 / 7.21, with the early exit 1.18 / 1.28;
 // 64^3, 1e3 0.47 / 0.54: only where both parts are large).  A launch pays for its last
 // wave, so where several classes would be launched a class of few items joins the finer
-// one before it (64^3, 1e3 sources of R = 5..50: one launch 0.52, three 0.87 ms), and
+// one before it (64^3, 1e3 sources of R = 5..50: one launch 0.52, three 0.87 ms), and two
+// quadrants per warp take many (128^3, two / one, batched and with the early exit: 900
+// sources of R = 27 0.542 / 0.520 and 0.204 / 0.141; 3e3 1.57 / 1.59 and 0.284 / 0.237), and
 // where one quadrant would take a warp longer than all work takes the GPU, CTAs trace
 // everything (64^3, 10 sources of R = 20: 0.048 against 0.057 ms; 128^3, 40 of R = 40:
 // 0.123 / 0.187).  With at most two items per SM they are the kAhead ones; with up to
@@ -345,7 +347,8 @@ static RatesPlan rates_plan(const Grid& g, const int* r2s, int ns, bool exit) {
   for (int k = K - 1; k > 1; --k) {
     double items = 24.0 / p.mode[k] * (p.cut[k + 1] - p.cut[k]);
     if (k == 2) items = std::min(items, 24.0 * (p.cut[2] - p.cut[1])) / (exit ? 6 : 2);
-    if (items < (p.cut[k] > 0 ? 6 : 1.2) * warps) p.cut[k] = p.cut[k + 1];
+    const double least = p.mode[k] == 2 ? (exit ? 30 : 8) : p.cut[k] > 0 ? 6 : 1.2;
+    if (items < least * warps) p.cut[k] = p.cut[k + 1];
   }
   return p;
 }
