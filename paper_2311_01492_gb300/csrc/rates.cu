@@ -575,9 +575,17 @@ __device__ __forceinline__ void flush_rates(const TraceArgs& a, unsigned nrate) 
   if ((threadIdx.x & 31) == 0 && nrate) atomicAdd(a.rate_cells, (unsigned long long)nrate);
 }
 
+// Threads per SM that the registers are cut for: 896 (72 registers) where all layers are
+// traced: 64 spill (250^3, 200 sources of R = 5..50: 0.323 / 0.260 ms; 128^3, 400: 0.395 /
+// 0.335), 80 leave too few CTAs (64^3, 256: 0.202 / 0.198 / 0.215); 1024 with the early
+// exit (128^3, 400: 0.067 / 0.071).
+constexpr int cta_threads(int what, bool ahead) {
+  return ahead ? 512 : what == RATES_EXIT ? 1024 : 896;
+}
+
 template <int BLOCK, int WHAT, bool AHEAD>
-__global__ void __launch_bounds__(BLOCK, (AHEAD ? 512 : 1024) / BLOCK) k_rates_cta(TraceArgs a,
-                                                                                int slots) {
+__global__ void __launch_bounds__(BLOCK, cta_threads(WHAT, AHEAD) / BLOCK)
+k_rates_cta(TraceArgs a, int slots) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_item;
   if (a.skip && *a.skip) return;
