@@ -285,8 +285,8 @@ static double longest_part(const Grid& g, int parts) {
 // Launches of the batched rates: sources [cut[k], cut[k+1]) (LPT order) by CTAs of
 // mode[0] threads (k = 0) or by warps with one quadrant, two, or a whole face (k > 0).
 struct RatesPlan {
-  static constexpr int kClasses = 5;
-  int mode[kClasses] = {128, 1, 1, 2, 4};
+  static constexpr int kClasses = 6;
+  int mode[kClasses] = {128, 1, 1, 2, 4, 4};
   int cut[kClasses + 1] = {};
 };
 
@@ -301,8 +301,9 @@ struct RatesPlan {
 // 5.57 and 0.75 / 0.71.  With optical-depth weights two never pay (2e3 sources of R =
 // 5..50: 2.77 ms with them, 2.54 without).  One quadrant per warp is launched twice, as its warps' shared memory goes by the widest source: from
 // half-width 30 on 14 warps fit an SM, below 21 (250^3, 3e5 sources of R = 5..50: 143.4 /
-// 138.2 ms in four launches; 128^3, 1.6e4 7.26 / 7.21, with the early exit 1.18 / 1.28;
-// 64^3, 1e3 0.47 / 0.54: only where both parts are large).  A launch pays for its last
+// 138.2 ms in four launches; 128^3, 1.6e4 7.26 / 7.21; 64^3, 1e3 0.47 / 0.54: only where
+// both parts are large); so are faces, from half-width 14 on (15 warps, below 21: 139.1 /
+// 135.9 ms; the 64-box ensemble 18.7 / 18.1; 250^3, 1e5 with the early exit 5.18 / 5.03).  A launch pays for its last
 // wave, so where several classes would be launched a class of few items joins the finer
 // one before it (64^3, 1e3 sources of R = 5..50: one launch 0.52, three 0.87 ms), and two
 // quadrants per warp take many (128^3, two / one, batched and with the early exit: 900
@@ -339,14 +340,16 @@ static RatesPlan rates_plan(const Grid& g, const int* r2s, int ns, bool exit) {
     for (int k = 1; k < K; ++k) p.cut[k] = ns;
     return p;
   }
-  const int face = g.ftab ? 16 : 0;
+  const int face = g.ftab ? 16 : 0, small = g.ftab ? 13 : 0;
   const bool od = g.interp_mode == RT_INTERP_OPTICAL_DEPTH;
   if (od) p.mode[3] = 1;
-  const int lim[K] = {0, exit && longest_part(g, 24) > 0.1 ? 19 : 38, 30, od ? face : 20, face};
+  const int lim[K] = {0, exit && longest_part(g, 24) > 0.1 ? 19 : 38, 30, od ? face : 20, face,
+                      small};
   for (int k = 1; k < K; ++k) p.cut[k] = std::max(p.cut[k - 1], first_fitting(g, r2s, ns, lim[k]));
   for (int k = K - 1; k > 1; --k) {
     double items = 24.0 / p.mode[k] * (p.cut[k + 1] - p.cut[k]);
-    if (k == 2) items = std::min(items, 24.0 * (p.cut[2] - p.cut[1])) / (exit ? 6 : 2);
+    if (p.mode[k] == p.mode[k - 1])
+      items = std::min(items, 24.0 / p.mode[k] * (p.cut[k] - p.cut[k - 1])) / 2;
     const double least = p.mode[k] == 2 ? (exit ? 30 : 8) : p.cut[k] > 0 ? 6 : 1.2;
     if (items < least * warps) p.cut[k] = p.cut[k + 1];
   }
