@@ -40,8 +40,8 @@ import numpy as np  # noqa: E402
 
 METRIC = "source-voxels/s (ns per source per voxel) at 250^3, ~1e6 src; batched vs plain"
 UNIT = "source-voxels/s"
-FP64_FLOPS_PER_SV = 9.0       # tau_in: 1 mul + 3 fma; tau_out: 1 fma
-FP64_FLOPS_PER_RATE = 10.0    # dtau*ds, 2 table fma, difference, 3 products
+FP64_FLOPS_PER_SV = 3.0       # scaled form: 1 add + 1 fma (its other two sums are integer)
+FP64_FLOPS_PER_RATE = 13.0    # weighted form instead (9 - 3), 2 table fma, difference, 2 products
 BYTES_PER_SV = 16.0           # dtau gather (8 B) + rate read-modify-write share (8 B)
 FP64_FMA_PER_CLK_SM, SM_MAX_GHZ = 2, 2.07   # GB300: 2 DFMA lanes per SM-cycle, 2.07 GHz max
 
@@ -140,7 +140,7 @@ class ClockSampler:
 def kernel_source_hash():
     import hashlib
     h = hashlib.sha256()
-    for f in ("trace.cu", "device_util.cuh"):
+    for f in ("rates.cu", "faces.cuh", "scaled_sum.cuh", "device_util.cuh"):
         with open(os.path.join(ROOT, "paper_2311_01492_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
@@ -536,7 +536,7 @@ def main():
                       "trace_ms": to, "ns_per_source_voxel": to * 1e6 / sv_sub,
                       "geometric_trace_ms": tn, "cost_over_geometric": to / tn,
                       "note": "labelled extra: interpolation weights w_n / max(tau_n, 0.6), "
-                              "normalised (four reciprocals and a division per cell)"}
+                              "normalised"}
         g.set_sources(pos_d, ndot_d, R_d)
 
     # ---------------- adjoint: gradient throughput, 1e5 sources of the same box
@@ -593,9 +593,13 @@ def main():
     hbm_gbs = BYTES_PER_SV * exact_sv / (tr_ms * 1e-3) / 1e9
     roofline = {"bound": "alu", "achieved": achieved_tf, "peak": peak_tf, "unit": "TFLOP/s",
                 "frac": achieved_tf / peak_tf, "traffic": traffic,
-                "kernel": "k_trace_faces + k_trace_faces_warp + k_trace_faces_whole_warp (the "
-                          "batched trace; FP64 pipe: %d SMs x 2 DFMA/clk x 2.07 GHz)" % sms,
+                "kernel": "k_rates_warp + k_rates_cta (the batched trace; FP64 pipe: %d SMs x "
+                          "2 DFMA/clk x 2.07 GHz)" % sms,
                 "algorithmic_flops_per_launch": flops,
+                # what the recurrence with bilinear weights (1 product, 4 fma a cell; 10 flops a
+                # rate) would have to sustain for the same time
+                "weighted_form_tflops": (9.0 * exact_sv + 10.0 * statistics.mean(rate_cells))
+                / (tr_ms * 1e-3) / 1e12,
                 "hbm_view": {"achieved_gbs": hbm_gbs, "peak_gbs": hbm_peak,
                              "frac": hbm_gbs / hbm_peak,
                              "target_frac": 0.5, "target_met": hbm_gbs / hbm_peak >= 0.5,

@@ -217,7 +217,7 @@ class Grid:
                 "rt_set_adjoint_mode")
 
     def set_schedule(self, block_big=128, hsmall=19, hface=13):
-        """Batched schedule: CTA size, warp-mode threshold, whole-face-warp threshold."""
+        """Batched schedule by thresholds (CTA size, warp mode, whole faces) instead of by rule."""
         L.check(self._lib.rt_set_schedule(self._h, int(block_big), int(hsmall), int(hface)),
                 "rt_set_schedule")
 

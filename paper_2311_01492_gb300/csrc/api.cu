@@ -296,10 +296,11 @@ struct RatesPlan {
 // R = 22 (15), 1e4: 7.4 / 4.7 / 4.0 / 3.7; R = 27 (19), 8e3: 7.7 / 5.1 / 4.7 / 5.8;
 // R = 33 (23), 5e3: 6.5 / 4.8 / 4.6 / -; R = 50 (35), 2e3: 5.8 / 5.3 / 7.0 / -; R = 60
 // (42), 1e3: 4.8 / 5.3 / - / -: hence the half-widths, but for two quadrants: since one
-// runs 21 warps per SM it takes at R = 33 what two take (4.22 / 4.28), in an ionised box
+// runs up to 24 warps per SM it takes at R = 33 what two take (4.22 / 4.28), in an ionised box
 // (1.5e3 sources) 4.88 / 5.62, with the early exit 0.41 / 0.45; at R = 27 5.17 / 5.03, 5.51 /
 // 5.57 and 0.75 / 0.71.  With optical-depth weights two never pay (2e3 sources of R =
-// 5..50: 2.77 ms with them, 2.54 without).  One quadrant per warp is launched twice, as its warps' shared memory goes by the widest source: from
+// 5..50: 2.77 ms with them, 2.54 without).  One quadrant per warp is launched twice, as
+// its warps' shared memory goes by the widest source: from
 // half-width 30 on 14 warps fit an SM, below 21 (250^3, 3e5 sources of R = 5..50: 143.4 /
 // 138.2 ms in four launches; 128^3, 1.6e4 7.26 / 7.21; 64^3, 1e3 0.47 / 0.54: only where
 // both parts are large); so are faces, from half-width 14 on (15 warps, below 21: 139.1 /

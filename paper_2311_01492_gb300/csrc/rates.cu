@@ -614,10 +614,10 @@ __host__ __device__ inline size_t warp_slots(int h, int mode) {
 }
 
 // Threads of a CTA and CTAs per SM that the registers are cut for.  The scaled part waits
-// for loads and shared memory, so warps count: with 16 (127 registers), 20 (96) or 21 (90)
-// per SM a batched trace of 128^3 takes, in one quadrant per warp (half-width 23, 5e3
+// for loads and shared memory, so warps count: with up to 16 (127 registers), 20 (96) or 24
+// (80) per SM a batched trace of 128^3 takes, in one quadrant per warp (half-width 23, 5e3
 // sources) 4.76 / 4.41 / 4.28 ms, in whole faces (11, 2e4) 3.02 / 2.76 / 2.65, in two
-// quadrants (15, 2e4; 90 registers spill) 4.28 / 4.02 / 4.82.  With optical-depth weights
+// quadrants (19, 8e3; 80 registers spill) 4.28 / 4.02 / 4.82.  With optical-depth weights
 // 7.19 / 7.26 / 7.31, with rates everywhere 2.33 / 2.29 / 2.31: FP64-bound.
 __host__ __device__ constexpr int rates_warps(int mode, bool exit, bool od) {
   return od ? 8 : mode == 2 || (mode == 4 && exit) ? 4 : 3;

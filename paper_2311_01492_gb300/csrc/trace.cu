@@ -16,9 +16,9 @@
 // a CTA-wide barrier between shells, keeping the column densities of its
 // source in a private cube of global memory.
 //
-// k_trace_faces (RT_SCHED_BATCHED) is the GB300 schedule, here for a source's column
-// densities and for the rates with optical-depth-modulated weights (the rates with the
-// geometric weights, whose items are the same, are in rates.cu).  The interpolants of
+// k_trace_faces (RT_SCHED_BATCHED) is the GB300 schedule, here for column densities that
+// rates.cu's CTAs do not hold and for optical-depth-modulated weights where CTAs are wanted
+// (the other rates, whose items are the same, are in rates.cu).  The interpolants of
 // a cell whose dominant axis is d lie in the plane one step closer to the
 // source along d (Eq. raga, entry plane), so the cells with dominant axis d
 // and sign +-1 -- a square pyramid ("face") -- form layers m = 1, 2, ... that
