@@ -707,7 +707,7 @@ static rt_status set_field(rt_grid_t h, const double* d, bool density) {
   if (!d) return fail(RT_ERR_INVALID, std::string(who) + ": null field");
   Grid& g = *reinterpret_cast<Grid*>(h);
   g.pin[0] = 0;
-  TRY(launch_validate_fields(g, density ? d : nullptr, density ? nullptr : d));
+  TRY(launch_validate_field(g, d, density ? 1e12 : 1.0));
   TRY(cudaStreamSynchronize(g.stream));
   if (g.pin[0])
     return fail(RT_ERR_INVALID, density ? "rt_set_density: n_H must be finite, >= +0 and <= 1e12"

@@ -325,7 +325,7 @@ cudaError_t launch_precompute(Grid& g, int what, double* out, const int* skip = 
 cudaError_t launch_tau_to_coldens(Grid& g, double* coldens);
 // gamma += thick / n_HI where thick != 0
 cudaError_t launch_add_thick(Grid& g, double* gamma, const int* skip);
-cudaError_t launch_validate_fields(Grid& g, const double* nH, const double* xHI);
+cudaError_t launch_validate_field(Grid& g, const double* v, double top);  // to g.pin[0]
 cudaError_t launch_geometry(GeoEntry* geo, GeoRow* georow, double* kap, double tau_lim, int mmax,
                             cudaStream_t s);
 cudaError_t launch_trace_faces(Grid& g, const TraceArgs& a, int block, int grid, size_t smem,
