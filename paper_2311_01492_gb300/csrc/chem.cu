@@ -39,8 +39,8 @@ __device__ __forceinline__ double short_decay(double y) {
 // density iteration takes about five passes of, in general, an expm1 and two divisions.
 // A warp whose cells all decay short takes the form above; the choice is the warp's (lane
 // by lane, mixed warps would issue both sides).  ms a step, before -> after: 250^3 with
-// 1e6 sources 8.92 -> 3.68, nearly ionised with 1e5 9.49 -> 8.72; 101^3 with 777 sources
-// 0.750 -> 0.273.
+// 1e6 sources 8.92 -> 3.63, nearly ionised with 1e5 9.49 -> 7.38 (8.72 with the hardware's
+// divisions); 101^3 with 777 sources 0.750 -> 0.257.
 // COLL: C_H != 0.
 template <bool COLL>
 __global__ void k_chemistry(int64_t n, const double* __restrict__ nH, double inv_a3,
