@@ -11,6 +11,7 @@
 #include <unordered_map>
 
 #include "asora_internal.cuh"
+#include "box_limits.h"
 
 namespace asora {
 
@@ -455,7 +456,7 @@ static rt_status run_trace(Grid& g, double* gamma, double* coldens, const int* i
   TRY(cudaMemsetAsync(g.counters, 0, 64 + 8 * sizeof(int), g.stream));  // and the queues
   const bool od = a.interp_mode == RT_INTERP_OPTICAL_DEPTH;
   const bool rates = gamma && takes_rates_kernels(g, early_exit);
-  if (schedule != RT_SCHED_PLAIN && g.nmax > 1290)
+  if (schedule != RT_SCHED_PLAIN && g.nmax > kMaxBox32)
     return fail(RT_ERR_INVALID, "rt_raytrace: the batched schedule needs boxes of at most "
                                 "1290^3 cells (32-bit offsets); use RT_SCHED_PLAIN");
   if (schedule == RT_SCHED_PLAIN) {
@@ -800,7 +801,7 @@ rt_status rt_raytrace_source_coldens(rt_grid_t h, int src, double* d_coldens, in
   if (st != RT_OK) return st;
   TRY(launch_precompute(g, PRE_DTAU, d_coldens));
   const int hmax = face_hcap(g.max_r2, g.nmax);
-  if (schedule != RT_SCHED_PLAIN && g.interp_mode == RT_INTERP_GEOMETRIC && g.nmax <= 1290 &&
+  if (schedule != RT_SCHED_PLAIN && g.interp_mode == RT_INTERP_GEOMETRIC && g.nmax <= kMaxBox32 &&
       rates_smem_bytes(hmax, few_items_block(hmax)) <= 227 * 1024) {
     // 24 CTAs, their source looked up on the device, with room for the widest one:
     // nothing is asked back
@@ -1031,13 +1032,11 @@ rt_status rt_raytrace_backward(rt_grid_t h, const double* d_dL_dgamma, double* d
     g.dq_cap = g.nsrc;
   }
   TRY(cudaMemsetAsync(g.dq_merged, 0, g.nsrc * sizeof(double), g.stream));
-  // Whole faces by warps (k_bwd_faces): every source if the recompute may stop at opaque
-  // layers (what does not fit is left to the quadrant kernels, through a list on the
-  // device), else those whose layers all fit.  Quadrant items of large sources by
-  // 128-thread CTAs, the rest one per warp (as the trace, but with the warp-mode threshold
-  // capped at half-width 27: such a warp keeps two layers and its layer records in shared
-  // memory, and beyond 27 too few stay resident -- 1e5 sources of the 250^3 workload took
-  // 1.5x longer at 30).
+  // Whole faces by warps (k_bwd_faces) and quadrants (adjoint_plan).  Quadrant items of large
+  // sources by 128-thread CTAs, the rest one per warp (as the trace, but with the warp-mode
+  // threshold capped at half-width 27: such a warp keeps two layers and its layer records in
+  // shared memory, and beyond 27 too few stay resident -- 1e5 sources of the 250^3 workload
+  // took 1.5x longer at 30).
   const int ns = g.nsrc;
   const int* r2s = g.r2_sorted_h.data();
   const int hbig = face_hcap(g.max_r2, g.nmax);
@@ -1048,10 +1047,10 @@ rt_status rt_raytrace_backward(rt_grid_t h, const double* d_dL_dgamma, double* d
   // quadrant (64^3, 256 sources: CTAs 0.21, with warps 0.47).
   const bool tables = g.ftab && g.kap_mmax >= 1 && longest_part(g, 6) <= 0.3;
   const int hwarp = !g.explicit_schedule && longest_part(g, 24) > 1.2 ? 0 : std::min(g.hsmall, 27);
-  const int face_begin = !tables ? ns : exit ? 0 : first_fitting(g, r2s, ns, kBwdFaceHcap);
-  const bool leftover = tables && exit && hbig > kBwdFaceHcap;
-  const int quads = exit && tables ? (leftover ? ns : 0) : face_begin;  // sources of the quadrant kernels
-  const int split = std::min(quads, first_fitting(g, r2s, ns, hwarp));
+  const AdjointPlan plan = adjoint_plan(ns, g.nmax, tables, exit, hbig, kBwdFaceHcap, hwarp,
+                                        [&](int h) { return first_fitting(g, r2s, ns, h); });
+  const int face_begin = plan.face_begin, quads = plan.quads, split = plan.split;
+  const bool leftover = plan.leftover;
   BwdLaunch Lc, Lw, Lf;  // CTAs, warps, faces
   Lc.exit = Lw.exit = Lf.exit = exit;
   Lc.lcap = Lw.lcap = lcap;
