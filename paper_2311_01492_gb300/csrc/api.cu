@@ -1047,69 +1047,82 @@ rt_status rt_raytrace_backward(rt_grid_t h, const double* d_dL_dgamma, double* d
   // quadrant (64^3, 256 sources: CTAs 0.21, with warps 0.47).
   const bool tables = g.ftab && g.kap_mmax >= 1 && longest_part(g, 6) <= 0.3;
   const int hwarp = !g.explicit_schedule && longest_part(g, 24) > 1.2 ? 0 : std::min(g.hsmall, 27);
-  const AdjointPlan plan = adjoint_plan(ns, g.nmax, tables, exit, hbig, kBwdFaceHcap, hwarp,
-                                        [&](int h) { return first_fitting(g, r2s, ns, h); });
+  AdjointPlan plan;
+  BwdLaunch Lc, Lw, Lf;  // CTAs, warps, faces
+  int hw = 0, nfaces = 0;
+  size_t stack_c = 0;
+  const int hf = std::min(hbig, kBwdFaceHcap);
+  auto prepare = [&](bool faces) -> rt_status {  // launches, and memory for them
+    plan = adjoint_plan(ns, g.nmax, faces, exit, hbig, kBwdFaceHcap, hwarp,
+                        [&](int h) { return first_fitting(g, r2s, ns, h); });
+    Lc = Lw = Lf = BwdLaunch();
+    Lc.exit = Lw.exit = Lf.exit = exit;
+    Lc.lcap = Lw.lcap = lcap;
+    if (plan.split > 0) {
+      Lc.block = 128;
+      Lc.smem = bwd_smem_bytes(hbig, lcap);
+      if (Lc.smem > 227 * 1024)
+        return fail(RT_ERR_INVALID, "rt_raytrace_backward: radius too large for the shared-memory layers");
+      Lc.stack_cap = face_stack_cap(g.max_r2, g.nmax);
+      const int maxg = bwd_max_grid(Lc.smem, 128);
+      if (maxg <= 0) return fail(RT_ERR_CUDA, "rt_raytrace_backward: no occupancy");
+      Lc.grid = std::max(1, std::min(24 * plan.split, maxg));
+    }
+    hw = plan.split < plan.quads ? face_hcap(r2s[plan.split], g.nmax) : 0;
+    if (plan.split < plan.quads) {
+      Lw.block = 32;
+      Lw.smem = bwd_smem_bytes(hw, lcap) * 8;
+      Lw.stack_cap = face_stack_cap(r2s[plan.split], g.nmax);
+      const int maxg = bwd_max_grid(Lw.smem, 32);
+      if (maxg <= 0) return fail(RT_ERR_CUDA, "rt_raytrace_backward: no occupancy (warp mode)");
+      Lw.grid = std::max(1, std::min((24 * (plan.quads - plan.split) + 7) / 8, maxg));
+    }
+    nfaces = 6 * (ns - plan.face_begin);
+    if (nfaces > 0) {
+      Lf.block = 4;
+      Lf.stack_cap = (size_t)std::max(g.face_stack, 1);
+      int maxg = 0;
+      Lf.wpb = 1;
+      for (int cand = 8; cand >= 1; --cand) {
+        const int mg = bwd_max_grid(bwd_face_smem_bytes(hf) * cand, 4, cand);
+        if (mg * cand > maxg * Lf.wpb) {
+          maxg = mg;
+          Lf.wpb = cand;
+        }
+      }
+      if (maxg <= 0) return fail(RT_ERR_CUDA, "rt_raytrace_backward: no occupancy (faces)");
+      Lf.smem = bwd_face_smem_bytes(hf) * Lf.wpb;
+      Lf.grid = std::max(1, std::min((nfaces + Lf.wpb - 1) / Lf.wpb, maxg));
+      Lf.redo_cap = plan.leftover ? 24 * ns : 0;
+      Lf.split_src = plan.split;
+    }
+    stack_c = Lc.stack_cap * Lc.grid;
+    const size_t stack_w = Lw.stack_cap * Lw.grid * 8;
+    const size_t stack_f = Lf.stack_cap * Lf.grid * Lf.wpb;  // (before the others, in their place)
+    const size_t need = std::max(stack_c + stack_w, stack_f) * sizeof(double2);
+    if (need > g.bwd_stack_bytes) {
+      dev_free(g.bwd_stack);
+      g.bwd_stack = nullptr;
+      g.bwd_stack_bytes = 0;
+      TRY(dev_malloc(&g.bwd_stack, need));
+      g.bwd_stack_bytes = need;
+    }
+    const size_t redo = 2 * (size_t)Lf.redo_cap;
+    if (redo > g.bwd_redo_cap) {
+      dev_free(g.bwd_redo);
+      g.bwd_redo = nullptr;
+      g.bwd_redo_cap = 0;
+      TRY(dev_malloc(&g.bwd_redo, redo * sizeof(int)));
+      g.bwd_redo_cap = redo;
+    }
+    return RT_OK;
+  };
+  st = prepare(tables);
+  // The faces' list takes 192 bytes a source, which the quadrant kernels do without.
+  if (st == RT_ERR_OOM && nfaces > 0) st = prepare(false);
+  if (st != RT_OK) return st;
   const int face_begin = plan.face_begin, quads = plan.quads, split = plan.split;
   const bool leftover = plan.leftover;
-  BwdLaunch Lc, Lw, Lf;  // CTAs, warps, faces
-  Lc.exit = Lw.exit = Lf.exit = exit;
-  Lc.lcap = Lw.lcap = lcap;
-  if (split > 0) {
-    Lc.block = 128;
-    Lc.smem = bwd_smem_bytes(hbig, lcap);
-    if (Lc.smem > 227 * 1024)
-      return fail(RT_ERR_INVALID, "rt_raytrace_backward: radius too large for the shared-memory layers");
-    Lc.stack_cap = face_stack_cap(g.max_r2, g.nmax);
-    const int maxg = bwd_max_grid(Lc.smem, 128);
-    if (maxg <= 0) return fail(RT_ERR_CUDA, "rt_raytrace_backward: no occupancy");
-    Lc.grid = std::max(1, std::min(24 * split, maxg));
-  }
-  const int hw = split < quads ? face_hcap(r2s[split], g.nmax) : 0;
-  if (split < quads) {
-    Lw.block = 32;
-    Lw.smem = bwd_smem_bytes(hw, lcap) * 8;
-    Lw.stack_cap = face_stack_cap(r2s[split], g.nmax);
-    const int maxg = bwd_max_grid(Lw.smem, 32);
-    if (maxg <= 0) return fail(RT_ERR_CUDA, "rt_raytrace_backward: no occupancy (warp mode)");
-    Lw.grid = std::max(1, std::min((24 * (quads - split) + 7) / 8, maxg));
-  }
-  const int hf = std::min(hbig, kBwdFaceHcap);
-  const int nfaces = 6 * (ns - face_begin);
-  if (nfaces > 0) {
-    Lf.block = 4;
-    Lf.stack_cap = (size_t)std::max(g.face_stack, 1);
-    int maxg = 0;
-    Lf.wpb = 1;
-    for (int cand = 8; cand >= 1; --cand) {
-      const int mg = bwd_max_grid(bwd_face_smem_bytes(hf) * cand, 4, cand);
-      if (mg * cand > maxg * Lf.wpb) {
-        maxg = mg;
-        Lf.wpb = cand;
-      }
-    }
-    if (maxg <= 0) return fail(RT_ERR_CUDA, "rt_raytrace_backward: no occupancy (faces)");
-    Lf.smem = bwd_face_smem_bytes(hf) * Lf.wpb;
-    Lf.grid = std::max(1, std::min((nfaces + Lf.wpb - 1) / Lf.wpb, maxg));
-    Lf.redo_cap = leftover ? 24 * ns : 0;
-    Lf.split_src = split;
-  }
-  const size_t stack_c = Lc.stack_cap * Lc.grid, stack_w = Lw.stack_cap * Lw.grid * 8;
-  const size_t stack_f = Lf.stack_cap * Lf.grid * Lf.wpb;  // (before the others, in their place)
-  const size_t need = std::max(stack_c + stack_w, stack_f) * sizeof(double2);
-  if (need > g.bwd_stack_bytes) {
-    dev_free(g.bwd_stack);
-    g.bwd_stack = nullptr;
-    g.bwd_stack_bytes = 0;
-    TRY(dev_malloc(&g.bwd_stack, need));
-    g.bwd_stack_bytes = need;
-  }
-  if (leftover && (size_t)Lf.redo_cap * 2 > g.bwd_redo_cap) {
-    dev_free(g.bwd_redo);
-    g.bwd_redo = nullptr;
-    g.bwd_redo_cap = 0;
-    TRY(dev_malloc(&g.bwd_redo, (size_t)Lf.redo_cap * 2 * sizeof(int)));
-    g.bwd_redo_cap = (size_t)Lf.redo_cap * 2;
-  }
   TraceArgs a = base_args(g);
   a.items = g.items;
   // queue: [0] CTAs, [1] warps, [2] faces, [4], [5] items left over for the first two
