@@ -19,7 +19,7 @@ namespace asora {
 //   <x> = x0 + q ((G + n_e C_H) dt - x0 y),   x(t + dt) = x0 + m (... the same),  m = 1 - y q:
 // no division and no expm1.  Taken where x0 >= 2^-9 or y >= 2^-10: there the cancellation
 // in x_eq + (x0 - x_eq) m costs that form less than 3e-13, and the two agree to that;
-// elsewhere (nearly neutral and hardly lit) the general form keeps its bits.
+// elsewhere (nearly neutral and hardly lit) the general form, whose cancellation is as it is.
 // q: polynomial through its values at the nine Chebyshev points of [0, 1/4],
 // relative error 2.6e-18 (measured in 60 digits).
 constexpr double kShort = 0.25;
@@ -37,10 +37,10 @@ __device__ __forceinline__ double short_decay(double y) {
 
 // FP64 issue binds (48 bytes a cell would take 0.11 ms at 250^3): a cell's electron-
 // density iteration takes about five passes of, in general, an expm1 and two divisions.
-// A warp whose cells all decay short takes the form above; the choice is the warp's (lane
-// by lane, mixed warps would issue both sides).  ms a step, before -> after: 250^3 with
-// 1e6 sources 8.92 -> 3.63, nearly ionised with 1e5 9.49 -> 7.38 (8.72 with the hardware's
-// divisions); 101^3 with 777 sources 0.750 -> 0.257.
+// The choice is the cell's alone, so that its bits do not depend on where it lies; a warp
+// with cells of both kinds issues both sides.  ms a step, before the short form -> with it:
+// 250^3 with 1e6 sources 8.92 -> 3.67, nearly ionised with 1e5 9.49 -> 8.34; 101^3 with 777
+// sources 0.750 -> 0.268.  (Chosen by the warp: 3.58, 7.33, 0.263.)
 // COLL: C_H != 0.
 template <bool COLL>
 __global__ void k_chemistry(int64_t n, const double* __restrict__ nH, double inv_a3,
@@ -69,10 +69,9 @@ __global__ void k_chemistry(int64_t n, const double* __restrict__ nH, double inv
       const double num = COLL ? G + ne * C_H : G;
       double xa_new;
       decays = rate > 0.0;
-      brief = __all_sync(__activemask(),
-                         decays && __double2hiint(y) < __double2hiint(kShort) &&
-                             (__double2hiint(xs) >= __double2hiint(1.0 / 512) ||
-                              __double2hiint(y) >= __double2hiint(1.0 / 1024)));
+      brief = decays && __double2hiint(y) < __double2hiint(kShort) &&
+              (__double2hiint(xs) >= __double2hiint(1.0 / 512) ||
+               __double2hiint(y) >= __double2hiint(1.0 / 1024));
       if (brief) {
         const double q = short_decay(y);
         const double diff = fma(-xs, y, num * dt);
