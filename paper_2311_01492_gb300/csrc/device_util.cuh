@@ -94,10 +94,10 @@ __device__ __forceinline__ double od_interp_r(double w1, double w2, double w3, d
                                               double nz) {
   const double v1 = w1 * r1, v2 = w2 * r2, v3 = w3 * r3, v4 = w4 * r4;
   const double S = ((v1 + v2) + v3) + v4;
-  return quick_div(fma(v4, c4, fma(v3, c3, fma(v2, c2, fma(v1, c1, nz)))), S);
+  return exact_div(fma(v4, c4, fma(v3, c3, fma(v2, c2, fma(v1, c1, nz)))), S);
 }
 __device__ __forceinline__ double od_recip(double c, double tw0) {
-  return quick_recip(max_pos(c, tw0));
+  return exact_recip(max_pos(c, tw0));
 }
 __device__ __forceinline__ double od_interp(double w1, double w2, double w3, double w4, double c1,
                                             double c2, double c3, double c4, double tw0,

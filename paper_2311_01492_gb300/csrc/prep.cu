@@ -103,7 +103,7 @@ __global__ void k_tau_to_coldens(int64_t n, double sigma0, double* __restrict__ 
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
        t += (int64_t)gridDim.x * blockDim.x) {
     const double v = c[t];
-    if (bits_of(v)) c[t] = quick_div(v, sigma0);
+    if (bits_of(v)) c[t] = exact_div(v, sigma0);
   }
 }
 

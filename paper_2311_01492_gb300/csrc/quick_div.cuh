@@ -1,4 +1,5 @@
-// Quotients of doubles with most of the work off the FP64 unit.  Plain C++ as well, so that
+// Quotients of doubles with most of the work off the FP64 unit: quick_div and quick_recip,
+// and exact_div and exact_recip where the bits of a / b are wanted.  Plain C++ as well, so that
 // the arithmetic can be checked on the host.
 //
 // GB300 issues one FP64 warp instruction per 68-76 cycles, and a / b costs nine of them
@@ -77,6 +78,34 @@ ASORA_HD double quick_recip(double b) {
   if (!qd_middle((uint32_t)(bb >> 32))) return plain_div(1.0, b);
   const double r = recip44((uint32_t)(bb >> 32), (uint32_t)bb);
   return fma(fma(-b, r, 1.0), r, r);
+}
+
+// The quotient rounded correctly, as a / b gives it, for one more FP64 turn: the remainder
+// t = a - b s of the rounded quotient s is exact, and |t| <= b ulp(s) / 2 says that s is the
+// nearest (a quotient of doubles is never halfway, nor within an ulp below a power of two).
+// b's exponent is moved as an integer: for a and b as above nothing leaves the range.
+// Optical-depth weights (128^3, 2e3 sources) with quick_div 2.43 ms, with these 2.51.
+ASORA_HD bool qd_nearest(double t, double b, double s) {
+  const uint64_t down = 1076 - (dbl_bits(s) >> 52);
+  return (dbl_bits(t) & 0x7fffffffffffffffull) <= dbl_bits(b) - (down << 52);
+}
+
+ASORA_HD double exact_div(double a, double b) {
+  const uint64_t ab = dbl_bits(a), bb = dbl_bits(b);
+  if (!(qd_middle((uint32_t)(bb >> 32)) && (qd_middle((uint32_t)(ab >> 32)) || ab == 0)))
+    return plain_div(a, b);
+  const double r = recip44((uint32_t)(bb >> 32), (uint32_t)bb);
+  const double q = a * r;
+  const double s = fma(fma(-b, q, a), r, q);
+  return qd_nearest(fma(-b, s, a), b, s) ? s : plain_div(a, b);
+}
+
+ASORA_HD double exact_recip(double b) {
+  const uint64_t bb = dbl_bits(b);
+  if (!qd_middle((uint32_t)(bb >> 32))) return plain_div(1.0, b);
+  const double r = recip44((uint32_t)(bb >> 32), (uint32_t)bb);
+  const double s = fma(fma(-b, r, 1.0), r, r);
+  return qd_nearest(fma(-b, s, 1.0), b, s) ? s : plain_div(1.0, b);
 }
 
 }  // namespace asora
