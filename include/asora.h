@@ -200,7 +200,12 @@ rt_status rt_raytrace_backward(rt_grid_t g, const double* d_dL_dgamma, double* d
  * sigma0 N_HI) and tau_in = sum(w'_n tau_n) / sum(w'_n), both sums in the order
  * n = 1..4 of the geometric chain.  tau_weight_min finite and > 0 (0.6 is the
  * binding's default).  The adjoint supports the geometric weights only (rt_raytrace_backward
- * returns RT_ERR_INVALID otherwise).  RT_ERR_INVALID for other modes. */
+ * returns RT_ERR_INVALID otherwise).  RT_ERR_INVALID for other modes.
+ * The first call with RT_INTERP_OPTICAL_DEPTH allocates scratch for the batched rates (228 KB
+ * per SM; it does not end a capture under way elsewhere).  Without memory for it the call
+ * succeeds and slower kernels run.  The grid keeps it when the mode goes back, and gives it
+ * up where another allocation of the grid does not fit, unless a trace with these weights
+ * was captured into a caller's graph. */
 rt_status rt_set_interpolation(rt_grid_t g, int mode, double tau_weight_min);
 
 /* Adjoint recompute mode: with stop_at_opaque != 0 (default) each item's

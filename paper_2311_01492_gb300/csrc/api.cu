@@ -77,6 +77,24 @@ rt_status cuda_fail(cudaError_t e, const char* what) {
   return e == cudaErrorMemoryAllocation ? RT_ERR_OOM : RT_ERR_CUDA;
 }
 
+// Whether work given to the stream now is captured into a caller's graph (if in doubt: yes).
+static bool in_capture(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  const bool clear = cudaPeekAtLastError() == cudaSuccess;
+  if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  if (clear) cudaGetLastError();  // (an error that was there stays)
+  return true;
+}
+
+bool release_scratch(Grid& g) {
+  if (!g.od_scratch || g.od_captured || in_capture(g.stream)) return false;
+  cudaGetLastError();  // (of the allocation that failed)
+  dev_free(g.od_scratch);  // waits for what still uses it
+  g.od_scratch = nullptr;
+  ++g.epoch;  // a kept graph holds its address
+  return true;
+}
+
 static int isqrt_h(int64_t x) {
   if (x <= 0) return 0;
   int64_t r = (int64_t)std::sqrt((double)x);
@@ -119,12 +137,12 @@ static rt_status ensure_geometry(Grid& g, int mmax) {
   if (mmax <= g.geo_mmax) return RT_OK;
   GeoEntry* geo = nullptr;
   GeoRow* georow = nullptr;
-  TRY(dev_malloc(&geo, geo_count(mmax) * sizeof(GeoEntry)));
+  TRY(grid_malloc(g, &geo, geo_count(mmax) * sizeof(GeoEntry)));
   const int kmax = std::min(mmax, kKapMax);
   double* kap = nullptr;
   const size_t nkap = 4 * georow_count(kmax) + (size_t)(kmax + 1) * (kmax + 2);
-  cudaError_t e = dev_malloc(&georow, georow_count(mmax) * sizeof(GeoRow));
-  if (e == cudaSuccess) e = dev_malloc(&kap, nkap * sizeof(double));
+  cudaError_t e = grid_malloc(g, &georow, georow_count(mmax) * sizeof(GeoRow));
+  if (e == cudaSuccess) e = grid_malloc(g, &kap, nkap * sizeof(double));
   if (e == cudaSuccess) e = launch_geometry(geo, georow, kap, g.p.tau_lim, mmax, g.stream);
   if (e != cudaSuccess) {
     dev_free(geo);
@@ -247,7 +265,7 @@ static rt_status ensure_cube(Grid& g, int nsrc, int* out_grid, int* out_E) {
     dev_free(g.cube);
     g.cube = nullptr;
     g.cube_bytes = 0;
-    TRY(dev_malloc(&g.cube, need));
+    TRY(grid_malloc(g, &g.cube, need));
     g.cube_bytes = need;
   }
   *out_grid = grid;
@@ -680,8 +698,8 @@ rt_status rt_set_tables(rt_grid_t h, int kind, int E0, int E1, int bits, const d
     }
   }
   double2 *dg = nullptr, *dh = nullptr;
-  TRY(dev_malloc(&dg, S * sizeof(double2)));
-  cudaError_t e = dev_malloc(&dh, S * sizeof(double2));
+  TRY(grid_malloc(g, &dg, S * sizeof(double2)));
+  cudaError_t e = grid_malloc(g, &dh, S * sizeof(double2));
   if (e == cudaSuccess) e = cudaMemcpy(dg, gc.data(), S * sizeof(double2), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(dh, hc.data(), S * sizeof(double2), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
@@ -773,6 +791,8 @@ rt_status rt_raytrace(rt_grid_t h, double* d_gamma, int schedule) {
   TRY(cudaEventRecord(g.ev[0], g.stream));
   const bool rates = schedule != RT_SCHED_PLAIN &&
                      takes_rates_kernels(g, schedule == RT_SCHED_BATCHED_EXIT);
+  if (rates && g.interp_mode == RT_INTERP_OPTICAL_DEPTH && !g.od_captured)
+    g.od_captured = in_capture(g.stream);
   TRY(launch_precompute(g, rates ? PRE_THICK : PRE_INVN, d_gamma));
   TRY(cudaEventRecord(g.ev[1], g.stream));
   if (g.nsrc > 0) {
@@ -916,14 +936,15 @@ rt_status rt_iterate(rt_grid_t h, double* d_x, double dt_s, double alpha_H, doub
   if (!g.nH) return fail(RT_ERR_STATE, "rt_iterate: rt_set_density not called");
   const size_t bytes = g.ncell * sizeof(double);
   if (!g.xbuf) {
-    TRY(dev_malloc(&g.xbuf, bytes));
-    TRY(dev_malloc(&g.xavg, bytes));
-    TRY(dev_malloc(&g.xavg2, bytes));
-    TRY(dev_malloc(&g.xhi_int, bytes));
+    TRY(grid_malloc(g, &g.xbuf, bytes));
+    TRY(grid_malloc(g, &g.xavg, bytes));
+    TRY(grid_malloc(g, &g.xavg2, bytes));
+    TRY(grid_malloc(g, &g.xhi_int, bytes));
   }
   g.xHI = g.xhi_int;
   const int64_t limit = (int64_t)std::ceil(conv_frac * (double)g.ncell);
   cudaStream_t user = g.stream;
+  if (g.od_scratch && !g.od_captured) g.od_captured = in_capture(user);
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   rt_status st = RT_OK;
@@ -1028,7 +1049,7 @@ rt_status rt_raytrace_backward(rt_grid_t h, const double* d_dL_dgamma, double* d
     dev_free(g.dq_merged);
     g.dq_merged = nullptr;
     g.dq_cap = 0;
-    TRY(dev_malloc(&g.dq_merged, g.nsrc * sizeof(double)));
+    TRY(grid_malloc(g, &g.dq_merged, g.nsrc * sizeof(double)));
     g.dq_cap = g.nsrc;
   }
   TRY(cudaMemsetAsync(g.dq_merged, 0, g.nsrc * sizeof(double), g.stream));
@@ -1104,7 +1125,7 @@ rt_status rt_raytrace_backward(rt_grid_t h, const double* d_dL_dgamma, double* d
       dev_free(g.bwd_stack);
       g.bwd_stack = nullptr;
       g.bwd_stack_bytes = 0;
-      TRY(dev_malloc(&g.bwd_stack, need));
+      TRY(grid_malloc(g, &g.bwd_stack, need));
       g.bwd_stack_bytes = need;
     }
     const size_t redo = 2 * (size_t)Lf.redo_cap;
@@ -1112,7 +1133,7 @@ rt_status rt_raytrace_backward(rt_grid_t h, const double* d_dL_dgamma, double* d
       dev_free(g.bwd_redo);
       g.bwd_redo = nullptr;
       g.bwd_redo_cap = 0;
-      TRY(dev_malloc(&g.bwd_redo, redo * sizeof(int)));
+      TRY(grid_malloc(g, &g.bwd_redo, redo * sizeof(int)));
       g.bwd_redo_cap = redo;
     }
     return RT_OK;
@@ -1171,15 +1192,19 @@ rt_status rt_set_interpolation(rt_grid_t h, int mode, double tau_weight_min) {
   if (mode == RT_INTERP_OPTICAL_DEPTH && !g.od_scratch) {
     // Room for the reciprocals of every resident warp of rates.cu: no more than their layers
     // take of the SMs' shared memory.  Here once, so that a trace allocates nothing and may
-    // be captured; without it (no memory, a capture under way) trace.cu, which needs none.
+    // be captured; where it fails, trace.cu, which needs none.  Kept when the mode goes back
+    // (a caller's graph may hold it), but given up where the grid needs the memory
+    // (release_scratch).  A capture under way, on whatever stream, is none of this call's
+    // business: relaxed mode lets the allocation through without ending it.
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    cudaStreamIsCapturing(g.stream, &cap);
-    if (cap == cudaStreamCaptureStatusNone)
-      dev_malloc(&g.od_scratch, (size_t)sms * 228 * 1024);  // (null where it fails)
-    cudaGetLastError();
+    const bool clear = cudaPeekAtLastError() == cudaSuccess;
+    cudaStreamCaptureMode relaxed = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&relaxed);
+    const cudaError_t e = dev_malloc(&g.od_scratch, (size_t)sms * 228 * 1024);
+    cudaThreadExchangeStreamCaptureMode(&relaxed);
+    if (e != cudaSuccess && clear) cudaGetLastError();  // (an error that was there stays)
   }
   g.interp_mode = mode;
   g.tau_w0 = tau_weight_min;
@@ -1259,7 +1284,7 @@ rt_status rt_autotune(rt_grid_t h, const char* cache_path, int* h_block, int* h_
     return RT_OK;
   }
   double* gam = nullptr;
-  TRY(dev_malloc(&gam, g.ncell * sizeof(double)));
+  TRY(grid_malloc(g, &gam, g.ncell * sizeof(double)));
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -1349,7 +1374,7 @@ rt_status rt_autotune(rt_grid_t h, const char* cache_path, int* h_block, int* h_
   // (RT_SCHED_AUTO then takes the faster)
   if (st == RT_OK) {
     float tp = 0.f;
-    TRY(dev_malloc(&gam, g.ncell * sizeof(double)));
+    TRY(grid_malloc(g, &gam, g.ncell * sizeof(double)));
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     cudaEventRecord(e0, g.stream);

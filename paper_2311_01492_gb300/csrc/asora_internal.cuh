@@ -240,7 +240,8 @@ struct Grid {
                        // from byte 64 of kPinBytes: the ingest's arrays, if they fit
   std::map<std::array<int, 4>, std::pair<int, int>> occupancy;  // of the rate kernels
   double* cube = nullptr;       // shell-kernel scratch
-  double* od_scratch = nullptr; // reciprocals of the batched rates with mode 1
+  double* od_scratch = nullptr; // reciprocals of the batched rates with mode 1 (may be null)
+  bool od_captured = false;     // a caller's graph holds its address
   size_t cube_bytes = 0;
   int64_t* unconv = nullptr;    // iteration counters
   double* xbuf = nullptr;       // rt_iterate buffers
@@ -302,6 +303,16 @@ cudaError_t dev_free(void* p);
 template <class T>
 inline cudaError_t dev_malloc(T** p, size_t bytes) {
   return dev_malloc_raw(reinterpret_cast<void**>(p), bytes);
+}
+
+// Gives back the grid's memory that only makes a trace faster; false if it holds none.
+bool release_scratch(Grid& g);
+// An allocation of an existing grid: such memory makes room for it.
+template <class T>
+inline cudaError_t grid_malloc(Grid& g, T** p, size_t bytes) {
+  cudaError_t e = dev_malloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && release_scratch(g)) e = dev_malloc(p, bytes);
+  return e;
 }
 
 // Frees the source arrays and the ingest scratch (prep.cu).

@@ -427,7 +427,7 @@ static cudaError_t reserve_sources(Grid& g, size_t n) {
   };
   if (e == cudaSuccess) {
     parts();
-    e = dev_malloc(&w.arena, bytes);
+    e = grid_malloc(g, &w.arena, bytes);
     base = w.arena;
     if (base) parts();
   }
@@ -807,7 +807,7 @@ rt_status ensure_row_tables(Grid& g) {
     }                                           \
   } while (0)
   parts();
-  CK(dev_malloc(&g.tables, bytes));
+  CK(grid_malloc(g, &g.tables, bytes));
   parts();
   CK(cudaMemcpyAsync(g.tables, up.data(), up.size(), cudaMemcpyHostToDevice, s));
   if (nent > 0) {
