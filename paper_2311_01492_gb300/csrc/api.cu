@@ -935,12 +935,8 @@ rt_status rt_iterate(rt_grid_t h, double* d_x, double dt_s, double alpha_H, doub
   if (!g.have_tables) return fail(RT_ERR_STATE, "rt_iterate: rt_set_tables not called");
   if (!g.nH) return fail(RT_ERR_STATE, "rt_iterate: rt_set_density not called");
   const size_t bytes = g.ncell * sizeof(double);
-  if (!g.xbuf) {
-    TRY(grid_malloc(g, &g.xbuf, bytes));
-    TRY(grid_malloc(g, &g.xavg, bytes));
-    TRY(grid_malloc(g, &g.xavg2, bytes));
-    TRY(grid_malloc(g, &g.xhi_int, bytes));
-  }
+  for (double** p : {&g.xbuf, &g.xavg, &g.xavg2, &g.xhi_int})  // (a call may have got only some)
+    if (!*p) TRY(grid_malloc(g, p, bytes));
   g.xHI = g.xhi_int;
   const int64_t limit = (int64_t)std::ceil(conv_frac * (double)g.ncell);
   cudaStream_t user = g.stream;
