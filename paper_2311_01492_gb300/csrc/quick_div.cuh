@@ -3,9 +3,9 @@
 // the arithmetic can be checked on the host.
 //
 // GB300 issues one FP64 warp instruction per 68-76 cycles, and a / b costs nine of them
-// (refinements of a hardware seed).  Here the seed is carried to 44 bits on the FP32
+// (refinements of a hardware seed).  Here the seed is carried to 41 bits on the FP32
 // and integer units, which leaves a product, its remainder and one correction (Markstein
-// 1990): the result is (a / b)(1 + d), |d| < 2^-85, rounded once.  Measured in the kernel
+// 1990): the result is (a / b)(1 + d), |d| < 2^-82, rounded once.  Measured in the kernel
 // that adds a / b to a field of 250^3 cells: 350 -> 165 us (74 by its bytes); batched rates
 // with optical-depth weights (128^3, 2e3 sources): 4.31 -> 2.83 ms.
 #pragma once
@@ -37,13 +37,13 @@ inline uint32_t qd_round(float x) { return (uint32_t)llrintf(x); }
 inline float qd_seed(float x) { return ASORA_QD_SEED(x); }
 #endif
 
-// 1/b from below or above by less than 2^-43, for 2^-400 <= b < 2^400.  b = f 2^k, f in
+// 1/b from below or above by less than 2^-41, for 2^-400 <= b < 2^400.  b = f 2^k, f in
 // [1, 2); h: f's first 24 bits, l: the next 23, as a number in [0, 1).  s, a float below
 // 1/f (rcp.approx is within 2^-23, h adds 2^-23, the fused step 2^-24) and not below 1/2;
-// 1/f = s + s (1 - f s) (1 + ..), where 1 - f s < 2^-21 is formed in two fused steps.  The
+// 1/f = s + s (1 - f s) (1 + ..), where 1 - f s < 2^-20.8 is formed in two fused steps.  The
 // correction is added to the double s as an integer count of units of 2^-53: s is in
 // [1/2, 1), so the sum never leaves its binade except to become 1.
-ASORA_HD double recip44(uint32_t hi, uint32_t lo) {
+ASORA_HD double recip41(uint32_t hi, uint32_t lo) {
   const float h = qd_float(0x3f800000u | ((hi << 3) & 0x7ffff8u) | (lo >> 29));
   const float l = qd_float(0x3f800000u | ((lo << 3) >> 9)) - 1.0f;
   const float s0 = qd_seed(h);
@@ -68,7 +68,7 @@ ASORA_HD double quick_div(double a, double b) {
   const uint64_t ab = dbl_bits(a), bb = dbl_bits(b);
   if (!(qd_middle((uint32_t)(bb >> 32)) && (qd_middle((uint32_t)(ab >> 32)) || ab == 0)))
     return plain_div(a, b);
-  const double r = recip44((uint32_t)(bb >> 32), (uint32_t)bb);
+  const double r = recip41((uint32_t)(bb >> 32), (uint32_t)bb);
   const double q = a * r;
   return fma(fma(-b, q, a), r, q);
 }
@@ -76,36 +76,45 @@ ASORA_HD double quick_div(double a, double b) {
 ASORA_HD double quick_recip(double b) {
   const uint64_t bb = dbl_bits(b);
   if (!qd_middle((uint32_t)(bb >> 32))) return plain_div(1.0, b);
-  const double r = recip44((uint32_t)(bb >> 32), (uint32_t)bb);
+  const double r = recip41((uint32_t)(bb >> 32), (uint32_t)bb);
   return fma(fma(-b, r, 1.0), r, r);
 }
 
-// The quotient rounded correctly, as a / b gives it, for one more FP64 turn: the remainder
-// t = a - b s of the rounded quotient s is exact, and |t| <= b ulp(s) / 2 says that s is the
-// nearest (a quotient of doubles is never halfway, nor within an ulp below a power of two).
-// b's exponent is moved as an integer: for a and b as above nothing leaves the range.
-// Optical-depth weights (128^3, 2e3 sources) with quick_div 2.43 ms, with these 2.51.
-ASORA_HD bool qd_nearest(double t, double b, double s) {
-  const uint64_t down = 1076 - (dbl_bits(s) >> 52);
-  return (dbl_bits(t) & 0x7fffffffffffffffull) <= dbl_bits(b) - (down << 52);
+// The quotients rounded correctly, as a / b gives them.  With q the first approximation, t its
+// remainder and r the reciprocal, q + t r is within 2^-29 ulp of the quotient, so its rounding
+// can only be wrong next to a tie: where x = |t r| in units of ulp(q) is close to halfway between
+// whole numbers.  x < 2^12 is formed from 32 bits of t and r each, beside the last FP64 step:
+// frac is its fraction, too low by less than 2^16 of 2^32.  q within 2^12 ulps of a power of
+// two counts as close to a tie as well: the rounded quotient may have another ulp.
+// Batched rates with optical-depth weights (128^3, 2e3 sources; with rates everywhere; 58^3,
+// two sources), quick_div / these / the exact remainder of the rounded quotient instead of x:
+// 2.51 / 2.52 / 2.59 ms, 7.38 / 7.43 / 8.74 ms, 144 / 148 / 164 us.
+ASORA_HD uint32_t qd_top32(uint64_t x) { return 0x80000000u | (uint32_t)(x >> 21); }
+
+ASORA_HD bool qd_near_tie(double q, double t, double r) {
+  const uint64_t qb = dbl_bits(q), tb = dbl_bits(t), rb = dbl_bits(r);
+  const uint32_t p = (uint32_t)(((uint64_t)qd_top32(tb) * qd_top32(rb)) >> 32);
+  const int k = ((int)(tb >> 52) & 0x7ff) + (int)(rb >> 52) - (int)(qb >> 52) - 1023 + 52;
+  const uint32_t frac = (uint32_t)shr64((uint64_t)p << 16, 14 - k);  // x = p 2^(k - 30)
+  const bool edge = ((qb + 4096) & 0xfffffffffffffull) < 8192;
+  return edge || frac - 0x7ffe0000u < 0x40000u;
 }
 
 ASORA_HD double exact_div(double a, double b) {
   const uint64_t ab = dbl_bits(a), bb = dbl_bits(b);
-  if (!(qd_middle((uint32_t)(bb >> 32)) && (qd_middle((uint32_t)(ab >> 32)) || ab == 0)))
-    return plain_div(a, b);
-  const double r = recip44((uint32_t)(bb >> 32), (uint32_t)bb);
+  if (!(qd_middle((uint32_t)(bb >> 32)) && qd_middle((uint32_t)(ab >> 32)))) return plain_div(a, b);
+  const double r = recip41((uint32_t)(bb >> 32), (uint32_t)bb);
   const double q = a * r;
-  const double s = fma(fma(-b, q, a), r, q);
-  return qd_nearest(fma(-b, s, a), b, s) ? s : plain_div(a, b);
+  const double t = fma(-b, q, a);
+  return qd_near_tie(q, t, r) ? plain_div(a, b) : fma(t, r, q);
 }
 
 ASORA_HD double exact_recip(double b) {
   const uint64_t bb = dbl_bits(b);
   if (!qd_middle((uint32_t)(bb >> 32))) return plain_div(1.0, b);
-  const double r = recip44((uint32_t)(bb >> 32), (uint32_t)bb);
-  const double s = fma(fma(-b, r, 1.0), r, r);
-  return qd_nearest(fma(-b, s, 1.0), b, s) ? s : plain_div(1.0, b);
+  const double r = recip41((uint32_t)(bb >> 32), (uint32_t)bb);
+  const double t = fma(-b, r, 1.0);
+  return qd_near_tie(r, t, r) ? plain_div(1.0, b) : fma(t, r, r);
 }
 
 }  // namespace asora
