@@ -6,8 +6,9 @@
 // four quadrants.  An item is traced in two parts.
 //
 // While a layer has cells with tau_out below the tables' bound 2^E1, the recurrence
-// of trace.cu is evaluated as written there, so that every rate has the bits it has
-// in the other schedules.  Once every cell of a layer is beyond the bound, every
+// of trace.cu is evaluated as written there, so that every optical depth has the bits
+// it has in the other schedules (a rate differs in how its constant factors are
+// grouped).  Once every cell of a layer is beyond the bound, every
 // later tau_in (a convex combination plus non-negative increments) is too, and every
 // later rate is exactly 0: the early exit stops there, the full schedule goes on and
 // forms the remaining column densities in the scaled form below.
